@@ -21,7 +21,7 @@ void whiten_ozaki(cudaStream_t s, int naux, long long ncol, long long ld, const 
 void whiten_float_float(cudaStream_t s, int m, long long ncol, const double* Linv, double* Lff, double* A, double* B,
                         long long ld, bool restore_a);
 void coulomb_kernels_load();
-void whiten_fp64_inplace(cudaStream_t s, int m, long long ncol, const double* L, double* A, long long ld);
+void whiten_fp64_inplace(cudaStream_t s, int m, int n, const double* L, double* A, long long ld);
 
 namespace {
 
@@ -117,46 +117,90 @@ int fail(df_handle* h, const Error& e) {
 
 }  // namespace
 
-// Inverse of a lower-triangular block of at most 64 rows in place (row-major, leading dimension ld): the
-// block is read into shared memory, then one thread per column j forward-substitutes and writes column j
-// of the inverse (it reads back only values it wrote itself).
-__global__ void tri_inv_small_kernel(double* __restrict__ L, int m, long long ld) {
-    __shared__ double a[64][65];
-    const int j = threadIdx.x;
-    for (int r = 0; r < m; ++r)
-        if (j < m) a[r][j] = L[(long long)r * ld + j];
-    __syncthreads();
-    if (j >= m) return;
-    for (int i = 0; i < j; ++i) L[(long long)i * ld + j] = 0.0;
-    L[(long long)j * ld + j] = 1.0 / a[j][j];
-    for (int i = j + 1; i < m; ++i) {
-        double t = 0.0;
-        for (int k = j; k < i; ++k) t = fma(a[i][k], L[(long long)k * ld + j], t);
-        L[(long long)i * ld + j] = -t / a[i][i];
+// t / a from the correctly rounded reciprocal r of a: the second residual correction rounds the quotient
+// correctly (Markstein, IBM J. Res. Dev. 34, 111 (1990)) as long as nothing leaves the normal range; five
+// FP64 instructions instead of a division's dozen and more
+__device__ __forceinline__ double quotient(double t, double a, double r) {
+    double q = t * r;
+    q = fma(fma(-a, q, t), r, q);
+    return fma(fma(-a, q, t), r, q);
+}
+
+// One lower-triangular block of at most 64 rows of L (row-major, leading dimension ld) applied by forward
+// substitution, as 32 threads for 4 columns: lane = (column, group of rows g, g + 8, ..., g + 56), its 8 rows in
+// registers. Step k takes the quotient of row k and subtracts its multiple from the rows below, at most 8
+// multiply-adds a lane. On the FP64 pipe (64 clocks a warp instruction) one warp needs about 18 us, and 608
+// warps (2432 columns) run at once; a thread walking its column in memory took 64 x 64 / 2 dependent steps,
+// 0.27 ms for 822 columns. The operations on each element, and their order, are those of that walk, so are the
+// bits: the metric's conditioning shows every rounding of L^-1 in J and K.
+__device__ __forceinline__ void tri_solve_cols(const double (&a)[64][65], const double* rinv, int m, double (&z)[8],
+                                               int lane) {
+    const int g = lane & 7, base = lane & ~7;
+    for (int k = 0; k < m; ++k) {
+        double t = z[0];
+#pragma unroll
+        for (int q = 1; q < 8; ++q) t = (k >> 3) == q ? z[q] : t;
+        const double x = quotient(__shfl_sync(0xffffffffu, t, base + (k & 7)), a[k][k], rinv[k]);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int row = g + 8 * q;
+            if (q > (k >> 3) || (q == (k >> 3) && g > (k & 7))) z[q] = fma(-a[row][k], x, z[q]);
+            else if (row == k) z[q] = x;
+        }
     }
 }
 
-// Z <- L^-1 Z for a lower-triangular block of at most 64 rows (row-major, leading dimension ld) and the
-// m x ncol right-hand sides Z (leading dimension ldz): one thread per column, forward substitution.
-__global__ void tri_solve_small_kernel(const double* __restrict__ L, int m, long long ld, double* __restrict__ Z,
-                                       int ncol, long long ldz) {
-    __shared__ double a[64][65];
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) a[e / m][e % m] = L[(long long)(e / m) * ld + e % m];
-    __syncthreads();
-    const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= ncol) return;
-    for (int i = 0; i < m; ++i) {
-        double t = Z[(long long)i * ldz + j];
-        for (int k = 0; k < i; ++k) t = fma(-a[i][k], Z[(long long)k * ldz + j], t);
-        Z[(long long)i * ldz + j] = t / a[i][i];
+__device__ __forceinline__ void load_tri_block(const double* __restrict__ L, int m, long long ld, double (&a)[64][65],
+                                               double* rinv) {
+    for (int e = threadIdx.x; e < 64 * 64; e += blockDim.x) {
+        const int r = e >> 6, c = e & 63;
+        a[r][c] = (r < m && c <= r) ? L[(long long)r * ld + c] : (r == c ? 1.0 : 0.0);
     }
+    __syncthreads();
+    if (threadIdx.x < 64) rinv[threadIdx.x] = 1.0 / a[threadIdx.x][threadIdx.x];
+    __syncthreads();
+}
+
+// Z <- L^-1 Z for the m x ncol rows Z (leading dimension ldz); 16 columns per CTA
+__global__ void __launch_bounds__(128) tri_solve_block_kernel(const double* __restrict__ L, int m, long long ld,
+                                                              double* __restrict__ Z, int ncol, long long ldz) {
+    __shared__ double a[64][65];
+    __shared__ double rinv[64];
+    load_tri_block(L, m, ld, a, rinv);
+    const int lane = threadIdx.x & 31, g = lane & 7;
+    const int j = blockIdx.x * 16 + (threadIdx.x >> 5) * 4 + (lane >> 3);
+    double z[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) z[q] = (g + 8 * q < m && j < ncol) ? Z[(long long)(g + 8 * q) * ldz + j] : 0.0;
+    tri_solve_cols(a, rinv, m, z, lane);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        if (g + 8 * q < m && j < ncol) Z[(long long)(g + 8 * q) * ldz + j] = z[q];
+}
+
+// X[b] (64 x 64) = inverse of the b-th 64-row diagonal block of L (m x m, leading dimension ld), every block in
+// one launch: blockIdx.y the block, 16 columns per CTA
+__global__ void __launch_bounds__(128) tri_inv_blocks_kernel(const double* __restrict__ L, int m, long long ld,
+                                                             double* __restrict__ X) {
+    __shared__ double a[64][65];
+    __shared__ double rinv[64];
+    const int i0 = blockIdx.y * 64, rows = min(64, m - i0);
+    load_tri_block(L + (long long)i0 * ld + i0, rows, ld, a, rinv);
+    const int lane = threadIdx.x & 31, g = lane & 7;
+    const int j = blockIdx.x * 16 + (threadIdx.x >> 5) * 4 + (lane >> 3);
+    double z[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) z[q] = g + 8 * q == j ? 1.0 : 0.0;
+    tri_solve_cols(a, rinv, rows, z, lane);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) X[((long long)blockIdx.y * 64 + g + 8 * q) * 64 + j] = z[q];
 }
 
 // Z <- L^-1 Z (L lower triangular m x m, leading dimension ld; Z m x ncol, leading dimension ldz) by
 // recursion: Z1 <- L11^-1 Z1, Z2 <- Z2 - L21 Z1, Z2 <- L22^-1 Z2 (blocked forward substitution).
 void tri_solve_lower(cudaStream_t s, const double* L, int m, long long ld, double* Z, int ncol, long long ldz) {
     if (m <= 64) {
-        tri_solve_small_kernel<<<(ncol + 127) / 128, 128, 0, s>>>(L, m, ld, Z, ncol, ldz);
+        tri_solve_block_kernel<<<(ncol + 15) / 16, 128, 0, s>>>(L, m, ld, Z, ncol, ldz);
         DF_CHECK_LAUNCH();
         return;
     }
@@ -172,23 +216,24 @@ void tri_solve_lower(cudaStream_t s, const double* L, int m, long long ld, doubl
 // X21 = -L22^-1 (L21 L11^-1) is taken by forward substitution with L22 before L22 is inverted: multiplying
 // by the explicit L22^-1 instead left residuals |X L - I| a hundred times larger on an ill-conditioned
 // metric (condition number 5e11 at 8 waters), enough to move the SCF energy by 1e-6 Eh. T is scratch
-// of (m/2 + 64) x (m/2 + 64) doubles.
-void tri_inv_lower(cudaStream_t s, double* L, int m, long long ld, double* T) {
+// of (m/2 + 64) x (m/2 + 64) doubles, inv the inverses of the 64-row diagonal blocks from row i0 / 64 on
+// (a leaf copies its own). Bound by the chain of its launches and the FP64 pipe.
+void tri_inv_lower(cudaStream_t s, double* L, int m, long long ld, double* T, const double* inv) {
     if (m <= 64) {
-        tri_inv_small_kernel<<<1, 64, 0, s>>>(L, m, ld);
-        DF_CHECK_LAUNCH();
+        DF_CUDA(cudaMemcpy2DAsync(L, sizeof(double) * ld, inv, sizeof(double) * 64, sizeof(double) * m, m,
+                                  cudaMemcpyDeviceToDevice, s));
         return;
     }
     const int m1 = ((m / 2 + 63) / 64) * 64, m2 = m - m1;
     double* L11 = L;
     double* L21 = L + (long long)m1 * ld;
     double* L22 = L21 + m1;
-    tri_inv_lower(s, L11, m1, ld, T);
-    dgemm(s, false, false, m2, m1, m1, -1.0, L21, (int)ld, L11, (int)ld, 0.0, T, m1);    // -L21 L11^-1
-    tri_solve_lower(s, L22, m2, ld, T, m1, m1);                                         // X21 = L22^-1 T
+    tri_inv_lower(s, L11, m1, ld, T, inv);
+    dgemm_lower(s, m2, m1, m1, -1.0, L21, (int)ld, L11, (int)ld, 0.0, T, m1);            // -L21 L11^-1
+    tri_solve_lower(s, L22, m2, ld, T, m1, m1);                                          // X21 = L22^-1 T
     DF_CUDA(cudaMemcpy2DAsync(L21, sizeof(double) * ld, T, sizeof(double) * m1, sizeof(double) * m1, m2,
                               cudaMemcpyDeviceToDevice, s));
-    tri_inv_lower(s, L22, m2, ld, T);
+    tri_inv_lower(s, L22, m2, ld, T, inv + (long long)m1 * 64);
 }
 
 void build_B(df_handle* h, double tau, bool keep, int whitening) {
@@ -234,9 +279,13 @@ void build_B(df_handle* h, double tau, bool keep, int whitening) {
             // the row-major lower factor: zero its upper triangle, then invert by blocks
             zero_upper_kernel<<<(unsigned)(((long long)na * na + 255) / 256), 256, 0, s>>>(h->Linv.p, na);
             DF_CHECK_LAUNCH();
-            DevBuf<double> T;
+            const int nblk = (na + 63) / 64;
+            DevBuf<double> T, inv;
             T.alloc((size_t)((na / 2 + 63) / 64 * 64) * (size_t)(na / 2 + 64));
-            tri_inv_lower(s, h->Linv.p, na, na, T.p);
+            inv.alloc((size_t)nblk * 64 * 64);
+            tri_inv_blocks_kernel<<<dim3(4, nblk), 128, 0, s>>>(h->Linv.p, na, na, inv.p);
+            DF_CHECK_LAUNCH();
+            tri_inv_lower(s, h->Linv.p, na, na, T.p, inv.p);
             DF_CUDA(cudaStreamSynchronize(s));
         } else {
             size_t dws = 0, hws = 0;
@@ -276,7 +325,7 @@ void build_B(df_handle* h, double tau, bool keep, int whitening) {
             h->A3c.p = nullptr;
             h->A3c.n = 0;
         }
-        whiten_fp64_inplace(s, na, h->pk.row, h->Linv.p, h->B.p, h->pk.row);
+        whiten_fp64_inplace(s, na, h->n, h->Linv.p, h->B.p, h->pk.row);
     } else if (wenv && std::string(wenv) == "ff") {
         // float-float whitening on the FP32 pipes (selectable for comparison)
         h->B.alloc(rows);
@@ -335,13 +384,11 @@ void jk_dispatch(df_handle* h, const double* dD, const double* dC, int nocc, dou
                  int slices) {
     ensure_jk_buffers(h, nocc);
     coulomb_fp64(h, dD, dJ);
-    const int ldy = ((nocc + 31) / 32) * 32;
-    pad_occupied(h, dC, nocc, ldy);
     if (precision == DF_PREC_SPLIT)
         exchange_split(h, dC, nocc, slices, dK);
     else
-        exchange_fp64(h, nocc, dK);
-    h->timings_ms[16] = 6 + h->exchange_launches;   // J (pack, gamma, coulomb, split sum, unpack), pad C, K
+        exchange_fp64(h, dC, nocc, dK);
+    h->timings_ms[16] = 5 + h->exchange_launches;   // J (pack, gamma, coulomb, split sum, unpack), K
 }
 
 // K alone for m columns of occupied-like coefficients dC (n x m, device), FP64 or split
@@ -350,8 +397,7 @@ void exchange_only(df_handle* h, const double* dC, int m, int precision, int sli
     if (precision == DF_PREC_SPLIT) {
         exchange_split(h, dC, m, slices, dK);
     } else {
-        pad_occupied(h, dC, m, ((m + 31) / 32) * 32);
-        exchange_fp64(h, m, dK);
+        exchange_fp64(h, dC, m, dK);
     }
 }
 
@@ -816,7 +862,7 @@ void df_free(df_handle* h) {
     if (h->own_stream) cudaStreamDestroy(h->own_stream);
     // device buffers released here, while the handle's device is current (their destructors then find them empty)
     DevBuf<double>* bufs[] = {&h->d_atom_xyz, &h->d_atom_Z, &h->S, &h->T, &h->V, &h->H, &h->metric, &h->Linv,
-                              &h->A3c, &h->B, &h->Dw, &h->gamma, &h->Jp, &h->Y, &h->Kpart, &h->Cpad, &h->dD,
+                              &h->A3c, &h->B, &h->Dw, &h->gamma, &h->Jp, &h->Y, &h->Kpart, &h->dD,
                               &h->dC, &h->dJ, &h->dK, &h->X, &h->F, &h->Fx, &h->Dm, &h->C, &h->eps, &h->work1,
                               &h->work2, &h->work3, &h->diisF, &h->diisE, &h->diisB, &h->Dspin};
     for (auto* b : bufs) b->release();

@@ -153,7 +153,7 @@ struct df_handle {
     bool a3c_ready = false;            // A3c already holds (P|mu nu) (grouped integrals of a batch)
 
     // J/K work
-    dfhf::DevBuf<double> Dw, gamma, Jp, Y, Kpart, Cpad, dD, dC, dJ, dK;
+    dfhf::DevBuf<double> Dw, gamma, Jp, Y, Kpart, dD, dC, dJ, dK;
     dfhf::DevBuf<int2> ktiles;
     int nocc_alloc = 0;
     dfhf::SplitState* split = nullptr;
@@ -191,22 +191,29 @@ void build_B_batch(df_handle** hs, int n, double tau, bool keep, int whitening, 
 void rys_eval(const double* dT, int count, int n, double* dx, double* dw, cudaStream_t s);
 
 // FP64 dense kernels (dense.cu)
-// C = alpha * op(A) * op(B) + beta * C, row-major, op(X) = X or X^T
+// C = alpha * op(A) * op(B) + beta * C, row-major, op(X) = X or X^T; the bits do not depend on the tile
 void dgemm(cudaStream_t s, bool ta, bool tb, int m, int n, int k, double alpha, const double* A, int lda,
            const double* B, int ldb, double beta, double* C, int ldc);
-// C = alpha * Linv * A for lower-triangular Linv (m x m), A (m x ncol), lda = ldc = row stride
-void dtrmm_lower(cudaStream_t s, int m, long long ncol, const double* Linv, const double* A, double* C,
-                 long long ld);
+// C[b][m][n] = alpha sum_k A[b][m][k] B[k][n] + beta C[b][m][n] over all batches b; element strides for the
+// batch (aB, cB) and each index; aM or aK is 1
+void dgemm_rows(cudaStream_t s, long long batches, int M, int N, int K, double alpha, const double* A, long long aB,
+                long long aM, long long aK, const double* B, long long bK, long long bN, double beta, double* C,
+                long long cB, long long cM, long long cN);
+// dgemm (ta = tb = false) for B[i][j] = 0 where i < j
+void dgemm_lower(cudaStream_t s, int m, int n, int k, double alpha, const double* A, int lda, const double* B, int ldb,
+                 double beta, double* C, int ldc);
+// y = A x (m rows of length k, stride lda); y = x^T A (k rows, n columns)
+void dgemv_rows(cudaStream_t s, int m, long long k, const double* A, long long lda, const double* x, double* y);
+void dgemv_cols(cudaStream_t s, int k, long long n, const double* A, long long lda, const double* x, double* y);
 
 // J/K (jk.cu)
 void jk_fp64(df_handle* h, const double* dD, const double* dC, int nocc, double* dJ, double* dK);
 void ensure_jk_buffers(df_handle* h, int nocc);
 void coulomb_fp64(df_handle* h, const double* dD, double* dJ);
-void pad_occupied(df_handle* h, const double* dC, int nocc, int ldy);
-// Y_{P,mu i} = sum_nu B_{P,mu nu} C_{nu i} from the packed FP64 B (Y: naux x np x ldy)
-void y_transform_fp64(cudaStream_t s, const double* B, long long row, int nt, int naux, const double* Cp, int ldy,
-                      int ncol, double* Y);
-void exchange_fp64(df_handle* h, int nocc, double* dK);
+// Y[mu][P nocc + i] = sum_nu B_{P,mu nu} C_{nu i} from the packed FP64 B (Y: n rows of naux nocc; C: n x nocc)
+void y_transform_fp64(cudaStream_t s, const double* B, long long row, int n, int naux, const double* C, int nocc,
+                      double* Y);
+void exchange_fp64(df_handle* h, const double* dC, int nocc, double* dK);
 int k_splits(const df_handle* h);
 void unpack_rows(df_handle* h, const double* packed, int p0, int count, double* dout);
 

@@ -6,8 +6,8 @@
 //       auxiliary indices (summed over both orbital indices);
 //   (3) contractions with a density matrix into an auxiliary vector and back, and with a four-index
 //       matrix G into a new object.
-// Every operation is one FP64 GEMM over a reshaped view of the tensors (the first-index transformation one
-// GEMM per auxiliary row), on the handle's stream.
+// Every operation is one FP64 GEMM over a reshaped view of the tensors (the first-index transformation batched
+// over the auxiliary rows) or, with a density, a matrix-vector product, on the handle's stream.
 #include <algorithm>
 #include <climits>
 #include <memory>
@@ -25,17 +25,25 @@ namespace dfhf {
 
 namespace {
 
-// C = op(A) op(B) with the rows of C in blocks small enough for the GEMM grid (rows of C: m)
+// C = op(A) op(B) with the rows of C in blocks that an int counts (rows of C: m)
 void gemm_rows(cudaStream_t s, bool ta, bool tb, long long m, long long n, long long k, const double* A, long long lda,
                const double* B, long long ldb, double* C, long long ldc) {
     if (n > INT_MAX || k > INT_MAX || lda > INT_MAX || ldb > INT_MAX || ldc > INT_MAX)
         throw Error{DF_E_ARG, "density-fitting operation: a matrix dimension exceeds the GEMM's range"};
-    const long long block = 65535LL * 64;
+    const long long block = 1LL << 30;
     for (long long r0 = 0; r0 < m; r0 += block) {
         const long long mr = std::min(block, m - r0);
         const double* Ab = ta ? A + r0 : A + r0 * lda;   // op(A) rows r0.. are columns of a stored-transposed A
-        dgemm(s, ta, tb, (int)mr, (int)n, (int)k, 1.0, Ab, (int)lda, B, (int)ldb, 0.0, C + r0 * ldc, (int)ldc);
+        dgemm_rows(s, 1, (int)mr, (int)n, (int)k, 1.0, Ab, 0, ta ? 1 : lda, ta ? lda : 1, B, tb ? 1 : ldb, tb ? ldb : 1, 0.0,
+                   C + r0 * ldc, 0, ldc, 1);
     }
+}
+
+// a density's length, as a GEMM dimension (the objects' products share one range)
+long long vector_length(const df_tensor* I) {
+    const long long rs = (long long)I->nr * I->ns;
+    if (rs > INT_MAX) throw Error{DF_E_ARG, "density-fitting operation: a matrix dimension exceeds the GEMM's range"};
+    return rs;
 }
 
 df_tensor* new_tensor(df_handle* h, int naux, int nr, int ns) {
@@ -147,11 +155,11 @@ int df_op_transform(const df_tensor* I, int which, const double* M, int m_rows, 
         upload(h, dM, M, (long long)m_rows * m_cols);
         std::unique_ptr<df_tensor> t;
         if (which == 0) {
-            // I'_{g,ts} = sum_r M_rt I_{g,rs}: per auxiliary row M^T (nt x nr) I_g (nr x ns)
+            // I'_{g,ts} = sum_r I_{g,rs} M_rt: the rows (g, s) of every auxiliary row in one product with M
             t.reset(new_tensor(h, I->naux, m_cols, I->ns));
-            for (int g = 0; g < I->naux; ++g)
-                gemm_rows(s, true, false, m_cols, I->ns, I->nr, dM.p, m_cols, I->d.p + (long long)g * I->nr * I->ns,
-                          I->ns, t->d.p + (long long)g * m_cols * I->ns, I->ns);
+            const long long ns = I->ns;
+            dgemm_rows(s, I->naux, I->ns, m_cols, I->nr, 1.0, I->d.p, I->nr * ns, 1, ns, dM.p, m_cols, 1, 0.0, t->d.p,
+                       m_cols * ns, 1, ns);
         } else if (which == 1) {
             // I'_{g,rt} = sum_s I_{g,rs} M_st: (naux nr) x ns times ns x nt
             t.reset(new_tensor(h, I->naux, I->nr, m_cols));
@@ -208,11 +216,11 @@ int df_op_density_fit(const df_tensor* I, const double* M, double* D) {
     df_handle* h = I->h;
     return guarded(h, [&] {
         // D_g = sum_rs I_{g,rs} M_rs: naux x (nr ns) times (nr ns) x 1
-        const long long rs = (long long)I->nr * I->ns;
+        const long long rs = vector_length(I);
         DevBuf<double> dM, dD;
         upload(h, dM, M, rs);
         dD.alloc(I->naux);
-        gemm_rows(h->stream, false, false, I->naux, 1, rs, I->d.p, rs, dM.p, 1, dD.p, 1);
+        dgemv_rows(h->stream, I->naux, rs, I->d.p, rs, dM.p, dD.p);
         download(h, D, dD, I->naux);
     });
 }
@@ -222,11 +230,11 @@ int df_op_density_back(const df_tensor* I, const double* D, double* M) {
     df_handle* h = I->h;
     return guarded(h, [&] {
         // M_rs = sum_g D_g I_{g,rs}: 1 x naux times naux x (nr ns)
-        const long long rs = (long long)I->nr * I->ns;
+        const long long rs = vector_length(I);
         DevBuf<double> dD, dM;
         upload(h, dD, D, I->naux);
         dM.alloc((size_t)rs);
-        gemm_rows(h->stream, false, false, 1, rs, I->naux, dD.p, I->naux, I->d.p, rs, dM.p, rs);
+        dgemv_cols(h->stream, I->naux, rs, I->d.p, rs, dD.p, dM.p);
         download(h, M, dM, rs);
     });
 }

@@ -12,10 +12,7 @@
 
 namespace dfhf {
 
-void y_transform_fp64(cudaStream_t s, const double* B, long long row, int nt, int naux, const double* Cp, int ldy,
-                      int ncol, double* Y);
-void k_syrk_fp64(cudaStream_t s, const double* Y, int naux, int np, int ldy, int ncol, int nsplit,
-                 const int2* tiles, int ntiles, double* Kpart, int n, double* K);
+void k_syrk_fp64(cudaStream_t s, const double* Y, int n, int naux, int nocc, int nsplit, double* part, double* K);
 
 namespace {
 
@@ -92,18 +89,11 @@ __global__ void sum_splits_kernel(const double* __restrict__ part, int nsplit, l
     out[i] = s;
 }
 
-// Cpad[mu][i] = C[mu][i] for mu < n, i < nocc; zero elsewhere (np x ldy)
-__global__ void pad_c_kernel(const double* __restrict__ C, int n, int nocc, int np, int ldy, double* __restrict__ Cp) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)np * ldy) return;
-    const int mu = (int)(idx / ldy), i = (int)(idx % ldy);
-    Cp[idx] = (mu < n && i < nocc) ? C[(long long)mu * nocc + i] : 0.0;
-}
-
 constexpr int J_SPLIT = 8;
 
 }  // namespace
 
+// partial sums of the FP64 exchange over ranges of the auxiliary index
 int k_splits(const df_handle* h) {
     const int tiles = h->pk.nt * (h->pk.nt + 1) / 2;
     int s = (4 * 152 + tiles - 1) / tiles;
@@ -119,7 +109,7 @@ void ensure_jk_buffers(df_handle* h, int nocc) {
         h->dD.alloc((size_t)h->n * h->n);
         h->dJ.alloc((size_t)h->n * h->n);
         h->dK.alloc((size_t)h->n * h->n);
-        h->Kpart.alloc((size_t)k_splits(h) * pk.np * pk.np);
+        h->Kpart.alloc((size_t)k_splits(h) * h->n * h->n);
         // tile list for the exchange contraction: lower tile pairs
         std::vector<int2> tiles;
         for (int I = 0; I < pk.nt; ++I)
@@ -128,8 +118,6 @@ void ensure_jk_buffers(df_handle* h, int nocc) {
         DF_CUDA(cudaMemcpyAsync(h->ktiles.p, tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice, h->stream));
     }
     if (nocc > h->nocc_alloc) {
-        const int ldy = ((nocc + 31) / 32) * 32;
-        h->Cpad.alloc((size_t)pk.np * ldy);
         h->dC.alloc((size_t)h->n * nocc);
         h->nocc_alloc = nocc;
     }
@@ -162,31 +150,24 @@ void coulomb_fp64(df_handle* h, const double* dD, double* dJ) {
     }
 }
 
-void pad_occupied(df_handle* h, const double* dC, int nocc, int ldy) {
-    const long long tot = (long long)h->pk.np * ldy;
-    pad_c_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, h->stream>>>(dC, h->n, nocc, h->pk.np, ldy, h->Cpad.p);
-    DF_CHECK_LAUNCH();
-}
-
-void exchange_fp64(df_handle* h, int nocc, double* dK) {
+void exchange_fp64(df_handle* h, const double* dC, int nocc, double* dK) {
     const Packing& pk = h->pk;
     cudaStream_t s = h->stream;
-    const int ldy = ((nocc + 31) / 32) * 32;
     PhaseTimer t(h->sync_timing, 3);
     t.mark(0, s);
     h->exchange_launches = 3;   // Y transform, K contraction, K reduction
-    // Y (naux x np x ldy doubles): the split exchange's Y buffer when the handle has one large enough (8 bytes
-    // per element as well; both run in order on the handle's stream), else its own, allocated on first use
-    const size_t ny = (size_t)h->naux * pk.np * ldy;
+    // Y (n rows of naux nocc doubles): the split exchange's Y buffer when the handle has one large enough (8
+    // bytes per element as well; both run in order on the handle's stream), else its own, allocated on first use
+    const long long KL = (long long)h->naux * nocc;
+    const size_t ny = (size_t)KL * h->n;
     double* Y = split_y_buffer(h, (long long)ny);
     if (!Y) {
         if (h->Y.n < ny) h->Y.alloc(ny);
         Y = h->Y.p;
     }
-    y_transform_fp64(s, h->B.p, pk.row, pk.nt, h->naux, h->Cpad.p, ldy, nocc, Y);
+    y_transform_fp64(s, h->B.p, pk.row, h->n, h->naux, dC, nocc, Y);
     t.mark(1, s);
-    const int ntiles = pk.nt * (pk.nt + 1) / 2;
-    k_syrk_fp64(s, Y, h->naux, pk.np, ldy, nocc, k_splits(h), h->ktiles.p, ntiles, h->Kpart.p, h->n, dK);
+    k_syrk_fp64(s, Y, h->n, h->naux, nocc, k_splits(h), h->Kpart.p, dK);
     t.mark(2, s);
     if (t.on) {
         t.sync(2);
@@ -198,8 +179,7 @@ void exchange_fp64(df_handle* h, int nocc, double* dK) {
 void jk_fp64(df_handle* h, const double* dD, const double* dC, int nocc, double* dJ, double* dK) {
     ensure_jk_buffers(h, nocc);
     coulomb_fp64(h, dD, dJ);
-    pad_occupied(h, dC, nocc, ((nocc + 31) / 32) * 32);
-    exchange_fp64(h, nocc, dK);
+    exchange_fp64(h, dC, nocc, dK);
 }
 
 void unpack_rows(df_handle* h, const double* packed, int p0, int count, double* dout) {

@@ -1,11 +1,13 @@
 // Density-fitted closed-shell MP2 correlation energy (the paper lists MP2 among the programs on the
 // density-fitting utilities, section "Program features"), FP64 on the GPU from the handle's B:
 //   * Y_{P,mu i} = sum_nu B_{P,mu nu} C_{nu i} (eq. 1, first form; the FP64 half-transform of the exchange);
-//   * B^P_{ia} = sum_mu C_{mu a} Y_{P,mu i} (eq. 1 again, on the second index), stored as T[i][a][P];
+//   * B^P_{ia} = sum_mu C_{mu a} Y_{P,mu i} (eq. 1 again, on the second index), one product over all P, stored
+//     as T[i][a][P];
 //   * for each occupied i, V_{ia,jb} = sum_P B^P_{ia} B^P_{jb} for every j <= i in one product
 //     (eq. 2, second form);
 //   * E2 = sum_{ij ab} (ia|jb) [2 (ia|jb) - (ib|ja)] / (e_i + e_j - e_a - e_b), every orbital correlated,
-//     each pair's sum in one block (fixed order) and the pairs added on the host in a fixed order.
+//     summed per pair and 32 x 32 tile of (a, b) in one block (fixed order), these added on the host in a
+//     fixed order.
 #include <cmath>
 #include <vector>
 
@@ -15,44 +17,51 @@ namespace dfhf {
 
 namespace {
 
-inline unsigned nb256(long long n) { return (unsigned)((n + 255) / 256); }
+constexpr int MT = 32;   // tile of virtual orbitals in the pair energies
 
-// Bia[P][a][i] (P < naux, a < nvir, i < nocc) -> T[i][a][P]
-__global__ void ov_transpose_kernel(const double* __restrict__ Bia, int naux, int nvir, int nocc,
-                                    double* __restrict__ T) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long total = (long long)naux * nvir * nocc;
-    if (idx >= total) return;
-    const int P = (int)(idx % naux);
-    const long long r = idx / naux;
-    const int a = (int)(r % nvir);
-    const int i = (int)(r / nvir);
-    T[idx] = Bia[((long long)P * nvir + a) * nocc + i];
-}
-
-// pair energies of occupied i with every j <= i: V holds (ia|jb) at V[a][j nvir + b] (row stride ld);
-// pe[j] = f sum_ab V_ab (2 V_ab - V_ba) / (e_i + e_j - e_a - e_b), f = 2 for j < i (the pair (j, i) too)
+// pair energies of occupied i with every j <= i: V holds (ia|jb) at V[a][j nvir + b] (row stride ld). Block
+// (t, j) takes the tile pair t = (ta >= tb): with N_ab = 1 / (e_i + e_j - e_a - e_b) the elements ab and ba
+// together give N_ab 2 (V_ab^2 + V_ba^2 - V_ab V_ba), so each quotient is taken once; both tiles pass through
+// shared memory so that V_ba is read along its rows. pe[j ntp + t] = f x sum, f = 2 for j < i (the pair (j, i)
+// too). Bound by the quotients' FP64 work; a block per pair left most SMs idle (0.13 ms a launch at 4 waters).
 __global__ void __launch_bounds__(256) pair_energy_kernel(const double* __restrict__ V, long long ld, int i, int nocc,
                                                           int nvir, const double* __restrict__ eps,
                                                           double* __restrict__ pe) {
-    const int j = blockIdx.x;
+    __shared__ double P[MT][MT + 1], Q[MT][MT + 1];
+    __shared__ double part[8];
+    const int t = blockIdx.x, j = blockIdx.y;
+    int ta = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
+    while ((ta + 1) * (ta + 2) / 2 <= t) ++ta;
+    while (ta * (ta + 1) / 2 > t) --ta;
+    const int tb = t - ta * (ta + 1) / 2;
+    const int c = threadIdx.x & 31, r0 = threadIdx.x >> 5;
+    const double* v = V + (long long)j * nvir;
+    for (int r = r0; r < MT; r += 8) {
+        const int a = ta * MT + r, b = tb * MT + c;
+        P[r][c] = (a < nvir && b < nvir) ? v[(long long)a * ld + b] : 0.0;          // (ia|jb)
+        const int a2 = tb * MT + r, b2 = ta * MT + c;
+        Q[r][c] = (a2 < nvir && b2 < nvir) ? v[(long long)a2 * ld + b2] : 0.0;
+    }
+    __syncthreads();
     const double eij = eps[i] + eps[j];
     const double* ev = eps + nocc;
     double s = 0.0;
-    for (long long ab = threadIdx.x; ab < (long long)nvir * nvir; ab += blockDim.x) {
-        const int a = (int)(ab / nvir), b = (int)(ab % nvir);
-        const double vab = V[(long long)a * ld + (long long)j * nvir + b];
-        const double vba = V[(long long)b * ld + (long long)j * nvir + a];
-        s += vab * (2.0 * vab - vba) / (eij - ev[a] - ev[b]);
+    for (int r = r0; r < MT; r += 8) {
+        const int a = ta * MT + r, b = tb * MT + c;
+        if (a >= nvir || b >= nvir || (ta == tb && b > a)) continue;
+        const double x = P[r][c], y = Q[c][r];                                       // V_ab, V_ba
+        const double num = (ta == tb && a == b) ? x * x : 2.0 * (x * x + y * y - x * y);
+        s += num / (eij - ev[a] - ev[b]);
     }
-    __shared__ double sm[256];
-    sm[threadIdx.x] = s;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (c == 0) part[r0] = s;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) sm[threadIdx.x] += sm[threadIdx.x + o];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        double sum = 0.0;
+        for (int w = 0; w < 8; ++w) sum += part[w];
+        pe[(long long)j * gridDim.x + t] = (j < i ? 2.0 : 1.0) * sum;
     }
-    if (threadIdx.x == 0) pe[j] = (j < i ? 2.0 : 1.0) * sm[0];
 }
 
 }  // namespace
@@ -61,9 +70,7 @@ double mp2_energy(df_handle* h, const double* C_host, const double* eps_host, in
     const int n = h->n, naux = h->naux, nvir = nmo - nocc;
     const Packing& pk = h->pk;
     cudaStream_t s = h->stream;
-    const int ldy = ((nocc + 31) / 32) * 32;
-    ensure_jk_buffers(h, nocc);
-    DevBuf<double> Call, Cocc, Cvir, eps, Y, Bia, T, V, pe;
+    DevBuf<double> Call, Cocc, Cvir, eps, Y, T, V, pe;
     Call.alloc((size_t)n * nmo);
     Cocc.alloc((size_t)n * nocc);
     Cvir.alloc((size_t)n * nvir);
@@ -74,37 +81,29 @@ double mp2_energy(df_handle* h, const double* C_host, const double* eps_host, in
                               cudaMemcpyDeviceToDevice, s));
     DF_CUDA(cudaMemcpy2DAsync(Cvir.p, sizeof(double) * nvir, Call.p + nocc, sizeof(double) * nmo, sizeof(double) * nvir,
                               n, cudaMemcpyDeviceToDevice, s));
-    // Y = B C_occ over the padded orbital rows (rows beyond n are zero)
-    pad_occupied(h, Cocc.p, nocc, ldy);
-    Y.alloc((size_t)naux * pk.np * ldy);
-    y_transform_fp64(s, h->B.p, pk.row, pk.nt, naux, h->Cpad.p, ldy, nocc, Y.p);
-    // B^P_ia = C_vir^T Y_P for every P, then T[i][a][P]
-    Bia.alloc((size_t)naux * nvir * nocc);
-    for (int P = 0; P < naux; ++P)
-        dgemm(s, true, false, nvir, nocc, n, 1.0, Cvir.p, nvir, Y.p + (long long)P * pk.np * ldy, ldy, 0.0,
-              Bia.p + (long long)P * nvir * nocc, nocc);
-    Y.release();
-    T.alloc((size_t)naux * nvir * nocc);
-    ov_transpose_kernel<<<nb256((long long)naux * nvir * nocc), 256, 0, s>>>(Bia.p, naux, nvir, nocc, T.p);
-    DF_CHECK_LAUNCH();
-    Bia.release();
+    const long long KL = (long long)naux * nocc;
+    Y.alloc((size_t)KL * n);
+    y_transform_fp64(s, h->B.p, pk.row, n, naux, Cocc.p, nocc, Y.p);
+    // T[i][a][P] = sum_mu Y[mu][P nocc + i] C_vir[mu][a]: rows (P, i), every P in one product
+    T.alloc((size_t)KL * nvir);
+    dgemm_rows(s, naux, nocc, nvir, n, 1.0, Y.p, nocc, 1, KL, Cvir.p, nvir, 1, 0.0, T.p, 1, (long long)nvir * naux, naux);
     // rows of pair integrals: V = T_i T_{0..i}^T (nvir x (i + 1) nvir) and the pair energies of row i
+    const int nt = (nvir + MT - 1) / MT, ntp = nt * (nt + 1) / 2;
     V.alloc((size_t)nvir * nocc * nvir);
-    pe.alloc((size_t)nocc * nocc);
-    pe.zero(s);
+    pe.alloc((size_t)nocc * (nocc + 1) / 2 * ntp);
     for (int i = 0; i < nocc; ++i) {
         const long long ld = (long long)(i + 1) * nvir;
-        dgemm(s, false, true, nvir, (int)ld, naux, 1.0, T.p + (long long)i * nvir * naux, naux, T.p, naux, 0.0, V.p,
-              (int)ld);
-        pair_energy_kernel<<<i + 1, 256, 0, s>>>(V.p, ld, i, nocc, nvir, eps.p, pe.p + (long long)i * nocc);
+        dgemm_rows(s, 1, nvir, (int)ld, naux, 1.0, T.p + (long long)i * nvir * naux, 0, naux, 1, T.p, 1, naux, 0.0, V.p, 0,
+                   ld, 1);
+        pair_energy_kernel<<<dim3(ntp, i + 1), 256, 0, s>>>(V.p, ld, i, nocc, nvir, eps.p,
+                                                           pe.p + (long long)i * (i + 1) / 2 * ntp);
         DF_CHECK_LAUNCH();
     }
-    std::vector<double> host((size_t)nocc * nocc);
+    std::vector<double> host((size_t)nocc * (nocc + 1) / 2 * ntp);
     DF_CUDA(cudaMemcpyAsync(host.data(), pe.p, sizeof(double) * host.size(), cudaMemcpyDeviceToHost, s));
     DF_CUDA(cudaStreamSynchronize(s));
     double e2 = 0.0;
-    for (int i = 0; i < nocc; ++i)
-        for (int j = 0; j <= i; ++j) e2 += host[(size_t)i * nocc + j];
+    for (double v : host) e2 += v;
     return e2;
 }
 
