@@ -339,37 +339,41 @@ void pick_and_launch(cudaStream_t s, GemmArgs g, const TileKernel (&kernels)[NT]
     pick->launch(s, g, (unsigned)count_tiles(pick->shape, g, syrk));
 }
 
-// K[mu][nu] = sum over the partial sums in order, both triangles: a CTA per lower 32 x 32 tile, a thread per
-// element (the transposed half through shared memory). Bound by the latency of the partial sums' reads, eight in
-// flight (n = 100, 68 sums: 26 us with four elements a thread).
-__global__ void __launch_bounds__(1024) syrk_reduce_kernel(const double* __restrict__ part, int nsplit, int n,
-                                                           double* __restrict__ K) {
-    __shared__ double t[32][33];
-    int I = (int)((sqrt(8.0 * blockIdx.x + 1.0) - 1.0) * 0.5);
-    while ((I + 1) * (I + 2) / 2 <= (int)blockIdx.x) ++I;
-    while (I * (I + 1) / 2 > (int)blockIdx.x) --I;
-    const int J = (int)blockIdx.x - I * (I + 1) / 2;
-    const int c = threadIdx.x & 31, r = threadIdx.x >> 5;
+// K[mu][nu] = sum over the partial sums in order, both triangles: a CTA per 8 rows of a lower 32 x 32 tile, a
+// thread per element (the transposed part through shared memory). Bound by the latency of the partial sums'
+// reads, eight in flight (n = 100, 68 sums: 26 us on the ten CTAs of whole tiles).
+__global__ void __launch_bounds__(256) syrk_reduce_kernel(const double* __restrict__ part, int nsplit, int n,
+                                                          double* __restrict__ K) {
+    __shared__ double t[8][33];
+    const int tile = blockIdx.x >> 2, r8 = (blockIdx.x & 3) * 8;
+    int I = (int)((sqrt(8.0 * tile + 1.0) - 1.0) * 0.5);
+    while ((I + 1) * (I + 2) / 2 <= tile) ++I;
+    while (I * (I + 1) / 2 > tile) --I;
+    const int J = tile - I * (I + 1) / 2;
     const long long nn = (long long)n * n;
-    const int mu = I * 32 + r, nu = J * 32 + c;
-    double s = 0.0;
-    if (mu < n && nu <= mu) {
-        const double* p = part + (long long)mu * n + nu;
-        int q = 0;
-        for (; q + 8 <= nsplit; q += 8) {
-            double v[8];
+    {
+        const int c = threadIdx.x & 31, r = threadIdx.x >> 5;
+        const int mu = I * 32 + r8 + r, nu = J * 32 + c;
+        double s = 0.0;
+        if (mu < n && nu <= mu) {
+            const double* p = part + (long long)mu * n + nu;
+            int q = 0;
+            for (; q + 8 <= nsplit; q += 8) {
+                double v[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = p[(q + u) * nn];
+                for (int u = 0; u < 8; ++u) v[u] = p[(q + u) * nn];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) s += v[u];
+                for (int u = 0; u < 8; ++u) s += v[u];
+            }
+            for (; q < nsplit; ++q) s += p[q * nn];
+            K[(long long)mu * n + nu] = s;
         }
-        for (; q < nsplit; ++q) s += p[q * nn];
-        K[(long long)mu * n + nu] = s;
+        t[r][c] = s;
     }
-    t[r][c] = s;
     __syncthreads();
-    const int mt = I * 32 + c, nt = J * 32 + r;   // element (mt, nt) mirrored to row nt
-    if (mt < n && nt < mt) K[(long long)nt * n + mt] = t[c][r];
+    const int c = threadIdx.x & 7, r = threadIdx.x >> 3;
+    const int mu = I * 32 + r8 + c, nu = J * 32 + r;   // element (mu, nu) mirrored to row nu
+    if (mu < n && nu < mu) K[(long long)nu * n + mu] = t[c][r];
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -667,7 +671,7 @@ void k_syrk_fp64(cudaStream_t s, const double* Y, int n, int naux, int nocc, int
     GemmArgs g{Y, 0, KL, 1, nullptr, 1, 0, part, 0, n, 1, (unsigned)n, n, n, (int)KL, 1.0, 0.0, 1, 1, 0, naux};
     pick_and_launch(s, g, SYRK_TILES, true, 1, nsplit);
     const int nt = (n + 31) / 32;
-    syrk_reduce_kernel<<<nt * (nt + 1) / 2, 1024, 0, s>>>(part, nsplit, n, K);
+    syrk_reduce_kernel<<<2 * nt * (nt + 1), 256, 0, s>>>(part, nsplit, n, K);
     DF_CHECK_LAUNCH();
 }
 

@@ -441,34 +441,35 @@ __global__ void __launch_bounds__(256) split_y_kernel(const float2* __restrict__
 // Y (hi, lo) -> Ys over the contiguous contraction index k = P ldy + i (KL = naux ldy values per row mu), one
 // exponent per (mu, chunk of CH consecutive k): the operand layout of the tensor-core exchange contraction.
 // Tile-major: Ys[s][k / 64][mu][k % 64], so that one TMA box (128 rows x 64 k) is 16 KB of contiguous memory;
-// no padding between auxiliary rows; the tail of the last 64-block (k >= KL) is zero. Warp per (mu, chunk).
+// no padding between auxiliary rows; the tail of the last 64-block (k >= KL) is zero, and so are the columns
+// i >= cols, which Y does not hold. Warp per (mu, chunk), a lane two consecutive k of every 64: the chunk is read
+// once into registers (it was read twice, and written two bytes a lane). Bound by HBM: 8 bytes in, 2 S out per
+// element.
 template <int S>
-__global__ void __launch_bounds__(256) split_y_rows_kernel(const float2* __restrict__ Y, int np, int ldy, long long KL,
-                                                           int CH, bf16* __restrict__ Ys, int* __restrict__ Ye) {
+__global__ void __launch_bounds__(256) split_y_rows_kernel(const float2* __restrict__ Y, int np, int ldy, int cols,
+                                                           long long KL, bf16* __restrict__ Ys, int* __restrict__ Ye) {
+    constexpr int CH = exact_chunk<S>(), IT = CH / 64;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const long long nchk = (KL + CH - 1) / CH;
     if (warp >= nchk * np) return;
     const int mu = (int)(warp % np);
     const long long b = warp / np;
-    const long long k0 = b * CH, k1 = min(KL, k0 + CH);
+    const long long k0 = b * CH;
     const long long nkb = (KL + 63) / 64;
     const long long sstride = nkb * np * 64;
-    // the chunk's k run over auxiliary rows P0, P0 + 1, ...: one division per warp, then per-row segments
-    const long long P0 = k0 / ldy;
-    const int i0 = (int)(k0 - P0 * ldy);
+    float4 v[IT];
     float mx = 0.f;
-    {
-        long long k = k0, P = P0;
-        int i = i0;
-        while (k < k1) {
-            const int seg = (int)min((long long)(ldy - i), k1 - k);
-            const float2* y = Y + (P * np + mu) * ldy + i;
-            for (int j = lane; j < seg; j += 32) mx = fmaxf(mx, fabsf(y[j].x));
-            k += seg;
-            ++P;
-            i = 0;
+#pragma unroll
+    for (int t = 0; t < IT; ++t) {
+        const long long k = k0 + t * 64 + 2 * lane;    // k and k + 1 lie in one auxiliary row (ldy is even)
+        v[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k < KL) {
+            const long long P = KL <= 0x7fffffff ? (long long)((unsigned)k / (unsigned)ldy) : k / ldy;
+            const int i = (int)(k - P * ldy);
+            if (i < cols) v[t] = __ldcs(reinterpret_cast<const float4*>(Y + (P * np + mu) * ldy + i));
         }
+        mx = fmaxf(mx, fmaxf(fabsf(v[t].x), fabsf(v[t].z)));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -476,36 +477,22 @@ __global__ void __launch_bounds__(256) split_y_rows_kernel(const float2* __restr
     if (mx > 0.f) frexpf(mx, &e);   // |hi + lo| 2^-e <= 1 + 2^-24, so |m_1| <= 128 still holds
     if (lane == 0) Ye[b * np + mu] = e;
     const float sc = pow2f(-e);
-    long long k = k0, P = P0;
-    int i = i0;
-    while (k < k1) {
-        const int seg = (int)min((long long)(ldy - i), k1 - k);
-        const float2* y = Y + (P * np + mu) * ldy + i;
-        for (int j = lane; j < seg; j += 32) {
-            const float2 v = y[j];
-            const long long kk = k + j;
-            bf16* out = Ys + ((kk >> 6) * np + mu) * 64 + (kk & 63);
-            float r = v.x * sc;
-            float rl = v.y * sc;
 #pragma unroll
-            for (int s = 0; s < S; ++s) {
-                const float tt = r * 128.f;
-                const float m = rintf(tt);
-                r = (tt - m) + rl * 128.f;
-                rl = 0.f;
-                out[s * sstride] = __float2bfloat16_rn(m);
-            }
+    for (int t = 0; t < IT; ++t) {
+        const long long kb = b * IT + t;
+        if (kb >= nkb) break;
+        __nv_bfloat162* out = reinterpret_cast<__nv_bfloat162*>(Ys + (kb * np + mu) * 64) + lane;
+        float r0 = v[t].x * sc, l0 = v[t].y * sc, r1 = v[t].z * sc, l1 = v[t].w * sc;
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            const float t0 = r0 * 128.f, t1 = r1 * 128.f;
+            const float m0 = rintf(t0), m1 = rintf(t1);
+            r0 = (t0 - m0) + l0 * 128.f;
+            r1 = (t1 - m1) + l1 * 128.f;
+            l0 = l1 = 0.f;
+            out[s * (sstride / 2)] = __floats2bfloat162_rn(m0, m1);
         }
-        k += seg;
-        ++P;
-        i = 0;
     }
-    if (k1 == KL)   // the warps of the last chunk zero the tail of the last 64-block
-        for (long long kk = KL + lane; kk < nkb * 64; kk += 32) {
-            bf16* out = Ys + ((kk >> 6) * np + mu) * 64 + (kk & 63);
-#pragma unroll
-            for (int s = 0; s < S; ++s) out[s * sstride] = __float2bfloat16_rn(0.f);
-        }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -609,17 +596,16 @@ int packed_preference() {
 }  // namespace
 
 void y_split_tc(cudaStream_t s, int S, int N, const bf16* Bs, const int* Be, const bf16* Cs, const int* Ce, int naux,
-                int np, int ldy, float2* Y, int* err);
+                int np, int ldy, int cols, float2* Y, int* err);
 void y_split_tc_packed(cudaStream_t s, int S, int N, const bf16* Bs, const int* Be, const bf16* Cs, const int* Ce,
-                       int naux, int zrows, int np, int nB, int ldy, float2* Y, int* err);
-void k_split_tc(cudaStream_t s, int S, int N, const bf16* Ys, const int* Ye, int naux, int np, int ldy, int nsplit,
-                const int2* tiles128, int ntiles, float2* Kpart, int npt, int* err);
+                       int naux, int zrows, int np, int nB, int ldy, int cols, float2* Y, int* err);
+void k_split_tc(cudaStream_t s, int S, int N, const bf16* Ys, const int* Ye, int naux, int np, int ldy, int cols, int nsplit,
+                float2* Kpart, int npt, int* err);
 void k_tc_reduce(cudaStream_t s, const float2* Kpart, int nsplit, int npt, int n, double* K);
 
 struct SplitState {
     // tensor-core (tcgen05) path
     int* err = nullptr;          // device error word of the tcgen05 kernels
-    int2* tiles128 = nullptr;    // lower 128-tile pairs
     float2* Kpart_tc = nullptr;  // [nsplit_tc][npt][npt]
     int npt = 0, ntiles128 = 0, nsplit_tc = 0, kcap = 0;   // kcap: splits Kpart_tc has room for
     int ksplit_heur = 1;         // K split of the occupancy heuristic (about 4 CTAs per SM)
@@ -636,6 +622,7 @@ struct SplitState {
     int* Ye = nullptr;
     float2* Kpart = nullptr;
     int ldy = 0;
+    int cols = 0;                // columns that hold orbitals, rounded up to 16 (tensor-core kernels compute these)
     int ldy_cap = 0;             // occupied width the Cs, Ce, Y and Ys buffers were sized for
     long long ye_cap = 0;        // entries of Ye
     int kpart_cap = 0;           // splits Kpart has room for (mma.sync contraction)
@@ -667,7 +654,6 @@ void free_split(df_handle* h) {
     cudaFree(st->Ye);
     cudaFree(st->Kpart);
     cudaFree(st->err);
-    cudaFree(st->tiles128);
     cudaFree(st->Kpart_tc);
     delete st;
     h->split = nullptr;
@@ -739,9 +725,9 @@ void prepare_b(df_handle* h, SplitState* st) {
 }
 
 // ---- autotuner ----------------------------------------------------------------------------------
-// The tile width of the tensor-core Y kernel (32, 64 or 80 columns dividing ldy) and of the K kernel (32
-// or 64) are picked by timing the candidates on the call's own operands the first time a size bucket
-// (np, ldy, naux / 512, S) is met; the choice is kept for the process. Y is timed on the first auxiliary
+// The tile width of the tensor-core Y kernel (32, 48, 64 or 80 columns) and of the K kernel (32, 48 or 64)
+// are picked by timing the candidates on the call's own operands the first time a size bucket
+// (np, columns, naux / 512, S) is met; the choice is kept for the process. Y is timed on the first auxiliary
 // block (all rows when every slice is resident), K on the finished Y slices. Every width computes the
 // same values bit for bit; the K split over auxiliary blocks comes from the occupancy heuristic.
 struct TcChoice {
@@ -771,18 +757,21 @@ double time_once(cudaStream_t s, F&& launch) {
 void y_tc(df_handle* h, SplitState* st, int S, int N, int p0, int nb, float2* Yb) {
     if (st->packed)   // slices at the buffer's full row stride (the padding of every block stays zero)
         y_split_tc_packed(h->stream, S, N, st->Bs, st->Be + p0, st->Cs, st->Ce, nb, st->blocked ? st->pblk : h->naux,
-                          st->np, st->nB, st->ldy, Yb, st->err);
+                          st->np, st->nB, st->ldy, st->cols, Yb, st->err);
     else
-        y_split_tc(h->stream, S, N, st->Bs, st->Be + (long long)p0 * st->np, st->Cs, st->Ce, nb, st->np, st->ldy, Yb,
-                   st->err);
+        y_split_tc(h->stream, S, N, st->Bs, st->Be + (long long)p0 * st->np, st->Cs, st->Ce, nb, st->np, st->ldy,
+                   st->cols, Yb, st->err);
 }
 
 template <int S>
 int tune_y(df_handle* h, SplitState* st, int nb, float2* Yb) {
     double best_ms = 1e30;
     int best = 0;
-    for (int N : {80, 64, 32}) {
-        if (st->ldy % N) continue;
+    int seen = 0;
+    for (int N : {32, 48, 64, 80}) {
+        if (seen >= st->cols) break;                 // an earlier width already covers every column
+        if (N == 48 && st->cols <= 64) continue;     // one tile of 64, or of the columns there are, covers them
+        seen = N;
         const double ms = time_once(h->stream, [&] { y_tc(h, st, S, N, 0, nb, Yb); });
         if (ms < best_ms) {
             best_ms = ms;
@@ -807,10 +796,9 @@ void tune_k(df_handle* h, SplitState* st, TcChoice& best) {
     }
     // the half-tile width at the heuristic's split
     double best_ms = 1e30;
-    for (int N : {64, 32}) {
+    for (int N : {64, 48, 32}) {
         const double ms = time_once(s, [&] {
-            k_split_tc(s, S, N, st->Ys, st->Ye, naux, np, ldy, h0, st->tiles128, st->ntiles128, st->Kpart_tc,
-                       st->npt, st->err);
+            k_split_tc(s, S, N, st->Ys, st->Ye, naux, np, ldy, st->cols, h0, st->Kpart_tc, st->npt, st->err);
         });
         if (ms < best_ms) {
             best_ms = ms;
@@ -839,14 +827,14 @@ void run_split(df_handle* h, SplitState* st, const double* dC, int nocc, double*
     DF_CUDA(cudaFuncSetAttribute(y_split_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const bool tc = use_tensor_cores() && (S == 3 || S == 5);
     if (st->packed && !tc) throw Error{DF_E_ARG, "internal: B slice layout does not match the exchange kernels"};
-    const std::array<int, 4> key{np, ldy, (naux + 511) / 512, S};
+    const std::array<int, 4> key{np, tc ? st->cols : ldy, (naux + 511) / 512, S};
     TcChoice ch;
     bool have = !tc;
     // DFHF_TC_TILES="yN,kN,ksplit" fixes the choice (tests compare tilings; the results do not depend on it)
     if (const char* f = tc ? std::getenv("DFHF_TC_TILES") : nullptr) {
         TcChoice fc;
         if (std::sscanf(f, "%d,%d,%d", &fc.yN, &fc.kN, &fc.ksplit) == 3 && fc.ksplit >= 1 &&
-            (fc.yN == 32 || fc.yN == 64 || fc.yN == 80) && ldy % fc.yN == 0 && (fc.kN == 32 || fc.kN == 64)) {
+            (fc.yN == 32 || fc.yN == 48 || fc.yN == 64 || fc.yN == 80) && (fc.kN == 32 || fc.kN == 48 || fc.kN == 64)) {
             ch = fc;
             have = true;
         }
@@ -900,8 +888,8 @@ void run_split(df_handle* h, SplitState* st, const double* dC, int nocc, double*
     const long long nblk = tc ? ((long long)naux * ldy + exact_chunk<S>() - 1) / exact_chunk<S>()
                               : (naux + st->PB - 1) / st->PB;
     if (tc)
-        split_y_rows_kernel<S><<<nblocks(nblk * np * 32, 256), 256, 0, s>>>(st->Y, np, ldy, (long long)naux * ldy,
-                                                                           exact_chunk<S>(), st->Ys, st->Ye);
+        split_y_rows_kernel<S><<<nblocks(nblk * np * 32, 256), 256, 0, s>>>(st->Y, np, ldy, st->cols,
+                                                                           (long long)naux * ldy, st->Ys, st->Ye);
     else
         split_y_kernel<S><<<nblocks(nblk * np * 32, 256), 256, 0, s>>>(st->Y, naux, np, ldy, st->PB, st->Ys, ystr,
                                                                       st->Ye);
@@ -942,8 +930,7 @@ void run_split(df_handle* h, SplitState* st, const double* dC, int nocc, double*
         }
         h->timings_ms[15] = ch.kN;
         ev.mark(3, s);
-        k_split_tc(s, S, ch.kN, st->Ys, st->Ye, naux, np, ldy, ksplit, st->tiles128, st->ntiles128, st->Kpart_tc,
-                   st->npt, st->err);
+        k_split_tc(s, S, ch.kN, st->Ys, st->Ye, naux, np, ldy, st->cols, ksplit, st->Kpart_tc, st->npt, st->err);
         ev.mark(4, s);
         k_tc_reduce(s, st->Kpart_tc, ksplit, st->npt, h->n, dK);
     } else {
@@ -1029,12 +1016,16 @@ void exchange_split(df_handle* h, const double* dC, int nocc, int slices, double
             b_exponents(h, st);
         }
     }
+    const int cols = (nocc + 15) / 16 * 16;
+    if (cols != st->cols) {
+        // the tile choices were made for other columns
+        for (int q = 0; q <= SMAX; ++q) st->ch_y[q] = st->ch_k[q] = st->ch_split[q] = 0;
+        st->cols = cols;
+    }
     if (ldy != st->ldy) {
         DF_CUDA(cudaStreamSynchronize(h->stream));   // earlier builds may still read these buffers
         if (ldy > CHUNK_TILES * KT) throw Error{DF_E_ARG, "split exchange supports nocc <= 512"};
         st->ldy = ldy;
-        // the tile choices were made for the previous occupied width (a width need not divide the new one)
-        for (int q = 0; q <= SMAX; ++q) st->ch_y[q] = st->ch_k[q] = st->ch_split[q] = 0;
         st->PB = std::max(1, (CHUNK_TILES * KT) / ldy);
         const int nt = st->np / 64;
         const int ntiles = nt * (nt + 1) / 2;
@@ -1079,15 +1070,10 @@ void exchange_split(df_handle* h, const double* dC, int nocc, int slices, double
             DF_CUDA(cudaMemsetAsync(st->err, 0, sizeof(int), h->stream));
         }
         // tcgen05 K: lower 128-tile pairs (fixed by np), split over exponent blocks to fill the GPU
-        if (!st->tiles128) {
+        if (!st->npt) {
             const int nt128 = (int)((np + 127) / 128);
             st->npt = nt128 * 128;
             st->ntiles128 = nt128 * (nt128 + 1) / 2;
-            std::vector<int2> t128;
-            for (int I = 0; I < nt128; ++I)
-                for (int J = 0; J <= I; ++J) t128.push_back(make_int2(I, J));
-            DF_CUDA(cudaMalloc((void**)&st->tiles128, sizeof(int2) * t128.size()));
-            DF_CUDA(cudaMemcpy(st->tiles128, t128.data(), sizeof(int2) * t128.size(), cudaMemcpyHostToDevice));
         }
         st->nsplit_tc = std::max(1, std::min((4 * 152 + 2 * st->ntiles128 - 1) / (2 * st->ntiles128), (int)nchk));
         st->ksplit_heur = st->nsplit_tc;

@@ -1,17 +1,18 @@
 // Split-precision exchange on the 5th-generation tensor cores (tcgen05 + TMEM + TMA).
 //
-// Same arithmetic as split_k.cu (Ozaki slices, exact 512-element FP32 chunks, float-float drains), with
-// the products issued as tcgen05.mma kind::f16 (BF16 x BF16 -> FP32 in tensor memory):
-//   * one CTA owns an output tile of 128 rows x N columns; every Ozaki level L = s + t (0-based) has
-//     its own FP32 accumulator of N columns in TMEM (S levels, S * N <= 512 columns);
-//   * a producer thread streams K-steps of 64 elements with TMA (3-D tensor maps, 128-byte swizzle):
-//     the S B slices of a K-step (N x 64 each) once into one of two resident buffers, and the S A
-//     slices (128 x 64) through a ring of slots; every buffer is guarded by mbarriers;
-//   * one thread issues the MMAs: for A slice s, the B slices t < S - s in wide MMAs (4 k16 steps
-//     each), then commits the A slot back to the producer, and the B buffer after the K-step's last
-//     A slice; at every chunk boundary it commits to the epilogue and waits until TMEM is free;
+// Same arithmetic as split_k.cu (Ozaki slices, exact FP32 chunks, float-float drains), with the products issued
+// as tcgen05.mma kind::f16 (BF16 x BF16 -> FP32 in tensor memory):
+//   * a CTA works on output tiles of 128 rows x N columns; every Ozaki level L = s + t (0-based) has its own FP32
+//     accumulator of N columns in TMEM (S levels, S * N <= 512 columns);
+//   * a producer warp streams K-steps of 64 elements with TMA (3-D tensor maps, 128-byte swizzle): the S B slices
+//     of a K-step (N x 64 each) once into one of two resident buffers, and the S A slices (128 x 64) through a
+//     ring of slots; every buffer is guarded by mbarriers;
+//   * an issuing warp: for A slice s, the B slices t < S - s in wide MMAs (4 k16 steps each), then the A slot
+//     goes back to the producer, and the B buffer after the K-step's last A slice; a chunk begins once the
+//     epilogue has taken the sums of the one before;
 //   * four epilogue warps (one per 32 TMEM lanes) read the level sums with tcgen05.ld, scale them by the
-//     exact power of two 2^{e_row + e_col - 7 (L + 2)} and add them into per-thread float-float rows.
+//     exact power of two 2^{e_row + e_col - 7 (L + 2)} and add them into per-thread float-float rows, two
+//     elements per instruction (f32x2).
 // Every mbarrier wait is bounded by a clock budget; on expiry the kernel records DF_E_TIMEOUT in a flag,
 // waits (with the full budget) for the copies and MMAs it has already issued, releases its tensor memory and
 // returns.
@@ -25,8 +26,10 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 #include <cstdlib>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "ozaki.cuh"
@@ -47,7 +50,7 @@ constexpr int chunk_steps() {
 // A-slice ring slots (one 128 x 64 slice each): 4, or 3 where that lets two CTAs share an SM
 template <int S, int N>
 constexpr int ring_slots() {
-    return (S >= 7 && N <= 32) ? 3 : 4;
+    return (S >= 7 && N <= 32) || (S == 5 && N == 48) || (S == 3 && N == 64) ? 3 : 4;
 }
 constexpr long long WAIT_CYCLES = 4000000000LL;   // ~2 s at 2 GHz
 
@@ -78,6 +81,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, unsigned parity) {
 // cycles (WAIT_CYCLES unless the host shortened it). The waits that drain copies and MMAs already issued,
 // before the CTA leaves, always keep the full WAIT_CYCLES.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, int* err, long long budget) {
+    if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {
         if (clock64() - t0 > budget || *(volatile int*)err) {
@@ -86,6 +90,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, int* e
         }
     }
     return true;
+}
+
+// the same by a whole warp, with one result for all of its lanes (the code after it stays uniform, so that the
+// MMA's operands live in uniform registers)
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, unsigned parity, int* err, long long budget) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, budget));
+}
+__device__ __forceinline__ bool elect_one() {
+    unsigned p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
 }
 
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
@@ -139,49 +154,85 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
 
-__device__ __forceinline__ void tmem_ld16(unsigned taddr, float* v) {
-    unsigned r[16];
+// 16 accumulator columns of this warp's 32 lanes: the load is issued here, the registers hold it after tmem_wait
+__device__ __forceinline__ void tmem_ld16(unsigned taddr, unsigned (&r)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
           "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+// waits for the loads issued so far; the registers pass through so that no use moves above the wait
+__device__ __forceinline__ void tmem_wait(unsigned (&r)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :
+                 : "memory");
+}
+
+// pairs of floats (two per 64-bit register): every operation rounds each half as the scalar one does
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pack2(unsigned a, unsigned b) { return (f2)a | ((f2)b << 32); }
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ float lo_of(f2 a) { return __uint_as_float((unsigned)a); }
+__device__ __forceinline__ float hi_of(f2 a) { return __uint_as_float((unsigned)(a >> 32)); }
 
 __device__ __forceinline__ float pow2f(int e) { return e < -126 ? 0.f : __int_as_float((127 + min(e, 127)) << 23); }
 
 
-__device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float v) {
-    const float s = hi + v;
-    const float bb = s - hi;
-    const float err = (hi - (s - bb)) + (v - bb);
+// (hi, lo) += v sc by Knuth's TwoSum, sc a power of two (the product v sc is exact, so it folds into the
+// multiply-adds): s = hi + v sc, b = s - hi, lo += (hi - (s - b)) + (v sc - b), hi = s
+__device__ __forceinline__ void two_sum_acc(f2& hi, f2& lo, f2 v, f2 sc) {
+    const f2 m1 = 0xBF800000BF800000ull;   // (-1, -1)
+    const f2 s = fma2(v, sc, hi);
+    const f2 nb = fma2(s, m1, hi);         // hi - s = -b
+    const f2 u = fma2(add2(s, nb), m1, hi);
+    lo = add2(lo, add2(u, fma2(v, sc, nb)));
     hi = s;
-    lo += err;
 }
 
 // ------------------------------------------------------------------------------------------------
-// Work description. MODE 0 (Y = B C): CTA = (P, mu-tile, n-tile); K runs over nu (np), exponents
-// constant (row: Be[P][mu], column: Ce[i]). MODE 3 (Y = B C from the packed slices): B_P is stored as its
-// lower 128 x 128 tiles only, Bs[s][P][t][128][128] with t = I (I + 1) / 2 + J for I >= J (diagonal tiles
-// whole), one exponent per P (Be[P]); K-step blocks nu of J > I come from the stored tile (J, I) read as an
-// MN-major (transposed) operand. MODE 1 (K = sum Y Y^T): CTA = (split, lower tile pair,
-// column part), the split slowest so that the CTAs resident together stream the same range of the
-// contraction through L2; K runs over the contiguous index k = P ldy + i of the Y slices, stored tile-major
-// as Ys[s][k / 64][mu][k % 64] (one TMA box is 16 KB of contiguous memory; no padding between auxiliary
-// rows), one exact chunk per block of consecutive k with its own exponents Ye[block][mu], Ye[block][nu].
+// Work description. The kernel is persistent: a CTA takes the tiles blockIdx.x, blockIdx.x + gridDim.x, ... and
+// its rings run on across them, so that the next tile's loads and products overlap the last drain and the
+// output of the one before (a CTA per tile spent the time of about 8 K-steps on its start and end: at n = 832,
+// 13 K-steps a tile, two fifths of the kernel).
+// MODE 0 (Y = B C): tile = (128 of the rows P np + mu, column tile), column tile fastest; K runs over nu (np),
+// exponents constant (row: Be[P np + mu], column: Ce[i]). MODE 3 (Y = B C from the packed slices): tile = (P,
+// mu-tile, column tile); B_P is stored as its lower 128 x 128 tiles only, Bs[s][P][t][128][128] with
+// t = I (I + 1) / 2 + J for I >= J (diagonal tiles whole), one exponent per P (Be[P]); K-step blocks nu of J > I
+// come from the stored tile (J, I) read as an MN-major (transposed) operand. In both only the columns below
+// `cols` (the occupied orbitals rounded up to 16) are computed: full tiles of N and a narrower last one.
+// MODE 1 (K = sum Y Y^T): tile = (split, 128-row tile, column tile up to the row tile's end), the split slowest so that the CTAs
+// resident together stream the same range of the contraction through L2; K runs over the contiguous index
+// k = P ldy + i of the Y slices, stored tile-major as Ys[s][k / 64][mu][k % 64] (one TMA box is 16 KB of
+// contiguous memory; no padding between auxiliary rows), one exact chunk per block of consecutive k with its own
+// exponents Ye[block][mu], Ye[block][nu]; the 16-wide blocks with i >= cols are zero and take no product.
+// MODE 2 (whitening): tile = (row tile, column tile), the last row tiles (the longest sums) first.
 // ------------------------------------------------------------------------------------------------
 struct TcArgs {
-    int mode;
-    int naux, np, ldy, PB, nsplit;
+    int naux, np, ldy, nsplit;
+    int rows;                // MODE 0: naux np
+    int cols;                // MODE 0, 1, 3: columns of Y that are not identically zero (a multiple of 16)
     long long KL;            // MODE 1: naux * ldy, the length of the contraction
     int nkb;                 // MODE 1: 64-wide blocks of the contraction, ceil(KL / 64)
-    int ntiles;              // MODE 1: lower 128-tile pairs
+    int ntiles;              // MODE 1: tiles of one split
     const int* row_e;        // MODE 0: Be [naux][np]; MODE 1: Ye [nchunk][np]
     const int* col_e;        // MODE 0: Ce [ldy]
-    const int2* tiles;       // MODE 1: lower 128-tile pairs
     float2* out;             // MODE 0: Y [naux][np][ldy]; MODE 1: Kpart [nsplit][npt][npt]
     int npt;                 // MODE 1: padded dimension of Kpart (multiple of 128)
     int* err;
@@ -192,15 +243,77 @@ struct TcArgs {
     long long ldo;
     long long wait_cycles;   // budget of the pipeline waits (WAIT_CYCLES by default)
     int nB;                  // MODE 3: 128-row blocks of the packed tiles (np padded to 128 nB)
+    int total;               // tiles of the launch
 };
 
+// one tile: first row and column, its width, K-steps; MODE 0 and 3: auxiliary row; MODE 1: split, its first
+// chunk and K-step
+struct Tile {
+    int m0, n0, nw, ksteps, P, split, chunk0, kb0;
+};
+
+// MODE 1: column tiles of width N that row tile I takes (the lower triangle of 128-blocks)
+__host__ __device__ __forceinline__ int k_col_tiles(int I, int N) { return ((I + 1) * TM + N - 1) / N; }
+
 template <int S, int N, int MODE>
-__global__ void __launch_bounds__(192, 1) ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA,
-                                                          const __grid_constant__ CUtensorMap mapB, TcArgs args) {
+__device__ __forceinline__ Tile decode_tile(const TcArgs& args, int b) {
+    Tile t{0, 0, N, 0, 0, 0, 0, 0};
+    if (MODE == 0 || MODE == 3) {
+        const int nt = (args.cols + N - 1) / N;
+        t.n0 = (b % nt) * N;
+        t.nw = min(N, args.cols - t.n0);
+        b /= nt;
+        if (MODE == 0) {
+            t.m0 = b * TM;
+            t.ksteps = args.np / KS;
+        } else {
+            t.m0 = (b % args.nB) * TM;
+            t.P = b / args.nB;
+            t.ksteps = 2 * args.nB;
+        }
+    } else if (MODE == 2) {
+        const int ntn = args.ncols / N, mt = (args.naux + TM - 1) / TM;
+        t.m0 = (mt - 1 - b / ntn) * TM;               // row-tile major: the L^-1 tile is shared in L2
+        t.n0 = (b % ntn) * N;
+        t.ksteps = (min(args.naux, t.m0 + TM) + KS - 1) / KS;   // L^-1 is lower triangular
+    } else {
+        constexpr int CH = exact_chunk<S>();
+        t.split = b / args.ntiles;
+        b -= t.split * args.ntiles;
+        int I = 0;
+        for (int c; b >= (c = k_col_tiles(I, N)); ++I) b -= c;
+        t.m0 = I * TM;
+        t.n0 = b * N;
+        const long long nchk = (args.KL + CH - 1) / CH;
+        const long long c0 = nchk * t.split / args.nsplit, c1 = nchk * (t.split + 1) / args.nsplit;
+        t.chunk0 = (int)c0;
+        const long long k0 = c0 * CH, k1 = min(args.KL, c1 * CH);
+        t.kb0 = (int)(k0 / KS);                                  // chunks are K-step aligned
+        t.ksteps = (int)((k1 - k0 + KS - 1) / KS);
+    }
+    return t;
+}
+
+// Two CTAs share an SM where the accumulators take at most half of its tensor memory (S N <= 256 columns): one
+// drains while the other's products run. What bounds it (measured on a stream of MMAs alone): an MMA of width W
+// takes max(W / 2, (4096 + 32 W) / 128) clocks, arithmetic or the read of its shared-memory operands at 128 bytes
+// a clock, and the TMA writes of the streamed slices (16 KB of A and 128 N bytes of B per slice and K-step) share
+// that memory; so wider tiles do better, up to the 48 columns at which two CTAs still fit (5 slices: 94 % of the
+// pipe without the writes, against 84 % at 32). The issuing and the loading warp run their loops as whole warps
+// with one elected lane per instruction: the operands (descriptors, addresses, coordinates) then sit in uniform
+// registers. As one-lane branches each MMA cost about 100 clocks of register moves.
+// Measured, 5 slices at n = 1200, naux = 3288, 120 occupied: Y 18.8 -> 12.7 ms (1.47 PFLOP/s), K 10.6 -> 7.6 ms;
+// whitening at naux = 1644, 225280 columns: 23.8 -> 12.8 ms. Of that, at np = 1216: uniform issue 919 -> 1077
+// TFLOP/s (K 1035 -> 1250), uniform loads 1172 -> 1233, packed drains + 4 %, persistent tiles over flattened rows
+// 1233 -> 1346, 48-wide tiles 1442.
+template <int S, int N, int MODE>
+__global__ void __launch_bounds__(192, S * N <= 256 ? 2 : 1)
+    ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+                    const __grid_constant__ CUtensorMap mapB2, const TcArgs args) {
     constexpr int A_BYTES = TM * KS * 2;          // 16 KB
-    constexpr int B_BYTES = N * KS * 2;           // a multiple of 1024 (N a multiple of 16)
-    constexpr int BSET = S * B_BYTES;             // every B slice of one K-step
+    constexpr int BSET = S * N * KS * 2;          // every B slice of one K-step (a slice: a multiple of 1024 bytes)
     constexpr int NA = ring_slots<S, N>();
+    constexpr int CSTEPS = chunk_steps<S>();
     constexpr int NCOLS = S * N <= 32 ? 32 : (S * N <= 64 ? 64 : (S * N <= 128 ? 128 : (S * N <= 256 ? 256 : 512)));
     static_assert(S * N <= 512, "TMEM holds at most 512 accumulator columns");
     constexpr int MMA_SLICES = 256 / N;            // B slices per MMA (M = 128 allows N <= 256)
@@ -218,47 +331,10 @@ __global__ void __launch_bounds__(192, 1) ozaki_tc_kernel(const __grid_constant_
     uint64_t* mma_done = acc_empty + 1;
     unsigned* tmem_slot = (unsigned*)(mma_done + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     int* err = args.err;
     const long long wait = args.wait_cycles;
-
-    // ---- work decode -------------------------------------------------------------------------
-    int P = 0, m0 = 0, n0 = 0, split = 0;
-    int2 IJ = make_int2(0, 0);
-    int ksteps = 0;
-    int p0 = 0, kpp = 0;   // MODE 1: first chunk and first K-step of the split
-    if (MODE == 0 || MODE == 3) {
-        const int mt = MODE == 3 ? args.nB : (args.np + TM - 1) / TM;
-        const int nt = args.ldy / N;
-        int b = blockIdx.x;
-        const int ntile = b % nt;
-        b /= nt;
-        m0 = (b % mt) * TM;
-        P = b / mt;
-        n0 = ntile * N;
-        ksteps = MODE == 3 ? 2 * args.nB : args.np / KS;
-    } else if (MODE == 2) {
-        const int ntn = args.ncols / N;
-        m0 = (blockIdx.x / ntn) * TM;             // row-tile major: the L^-1 tile is shared in L2
-        n0 = (blockIdx.x % ntn) * N;
-        ksteps = (min(args.naux, m0 + TM) + KS - 1) / KS;   // L^-1 is lower triangular
-    } else {
-        const int halves = TM / N;
-        int b = blockIdx.x;
-        const int h = b % halves;
-        b /= halves;
-        IJ = args.tiles[b % args.ntiles];
-        split = b / args.ntiles;
-        m0 = IJ.x * TM;
-        n0 = IJ.y * TM + h * N;
-        constexpr int CH = exact_chunk<S>();
-        const long long nchk = (args.KL + CH - 1) / CH;
-        const long long c0 = nchk * split / args.nsplit, c1 = nchk * (split + 1) / args.nsplit;
-        p0 = (int)c0;                                              // first chunk of this split
-        const long long k0 = c0 * CH, k1 = min(args.KL, c1 * CH);
-        kpp = (int)(k0 / KS);                                      // first K-step (chunks are K-step aligned)
-        ksteps = (int)((k1 - k0 + KS - 1) / KS);
-    }
+    const int total = args.total;
 
     // ---- set-up: barriers (thread 0), tensor memory (warp 0) ------------------------------------
     if (threadIdx.x == 0) {
@@ -285,194 +361,278 @@ __global__ void __launch_bounds__(192, 1) ozaki_tc_kernel(const __grid_constant_
     fence_after();
     const unsigned tmem = *tmem_slot;
 
-    // chunk index of K-step ks (every mode: the exact chunk of S slices)
-    auto chunk_of = [&](int ks) { return ks / chunk_steps<S>(); };
-    const int nchunks = ksteps > 0 ? chunk_of(ksteps - 1) + 1 : 0;
-
     if (warp == 4) {
         // ---------------------------------- producer ------------------------------------------
-        if (lane == 0) {
-            asm volatile("prefetch.tensormap [%0];\n" ::"l"((unsigned long long)&mapA) : "memory");
-            asm volatile("prefetch.tensormap [%0];\n" ::"l"((unsigned long long)&mapB) : "memory");
-            int a_issued = 0, b_issued = 0;
-            for (int ks = 0; ks < ksteps; ++ks) {
+        const bool leader = elect_one();
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"((unsigned long long)&mapA) : "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"((unsigned long long)&mapB) : "memory");
+        int slot = 0, bs = 0;
+        unsigned aph = 0, bph = 0;                // ring phases
+        int a_issued = 0, b_issued = 0;           // capped counts: which buffers have copies to wait for
+        bool ok = true;
+        for (int b = blockIdx.x; b < total && ok; b += gridDim.x) {
+            const Tile t = decode_tile<S, N, MODE>(args, b);
+            const CUtensorMap* mb = t.nw == N ? &mapB : &mapB2;
+            const int bslice = t.nw * KS * 2;
+            for (int ks = 0; ks < t.ksteps && ok; ++ks) {
                 // x: the contraction coordinate of this K-step; MODE 1 reads the tile-major slices
                 // [s][k block][row][64] at x = 0 and z = s nkb + the split's K-step
                 const int kx = MODE == 1 ? 0 : ks * KS;
-                const int kb = kpp + ks;
-                const int bs = ks & 1;
-                if (!mbar_wait(&b_empty[bs], ((ks >> 1) & 1) ^ 1, err, wait)) break;
-                mbar_expect_tx(&b_full[bs], BSET);
-                for (int t = 0; t < S; ++t)
-                    tma_load_3d(bbuf + bs * BSET + t * B_BYTES, &mapB, kx, n0, MODE == 1 ? t * args.nkb + kb : t,
-                                &b_full[bs]);
-                ++b_issued;
-                bool ok = true;
+                const int kb = t.kb0 + ks;
+                if (!(ok = mbar_wait_warp(&b_empty[bs], bph ^ 1, err, wait))) break;
+                if (leader) {
+                    mbar_expect_tx(&b_full[bs], S * bslice);
+#pragma unroll
+                    for (int q = 0; q < S; ++q)
+                        tma_load_3d(bbuf + bs * BSET + q * bslice, mb, kx, t.n0, MODE == 1 ? q * args.nkb + kb : q,
+                                    &b_full[bs]);
+                }
+                b_issued = min(b_issued + 1, 2);
+                bs ^= 1;
+                if (bs == 0) bph ^= 1;
+#pragma unroll
                 for (int s = 0; s < S; ++s) {
-                    const int it = ks * S + s, slot = it % NA;
-                    if (!mbar_wait(&a_empty[slot], ((it / NA) & 1) ^ 1, err, wait)) {
-                        ok = false;
-                        break;
-                    }
-                    mbar_expect_tx(&a_full[slot], A_BYTES);
-                    const int za = (MODE == 0 || MODE == 3) ? s * args.naux + P : (MODE == 1 ? s * args.nkb + kb : s);
-                    if (MODE == 3) {
-                        // two 64-row boxes of one stored tile: rows mu of tile (I, J) at columns nu of this
-                        // K-step (K-major), or, above the diagonal, rows nu of tile (J, I) (MN-major halves)
-                        const int I = m0 / TM, J = ks >> 1, half = ks & 1;
+                    if (!(ok = mbar_wait_warp(&a_empty[slot], aph ^ 1, err, wait))) break;
+                    if (leader) {
+                        mbar_expect_tx(&a_full[slot], A_BYTES);
                         unsigned char* dst = smem + slot * A_BYTES;
-                        if (I >= J) {
-                            const int y0 = (I * (I + 1) / 2 + J) * TM;
-                            tma_load_3d(dst, &mapA, half * KS, y0, za, &a_full[slot]);
-                            tma_load_3d(dst + A_BYTES / 2, &mapA, half * KS, y0 + KS, za, &a_full[slot]);
+                        if (MODE == 3) {
+                            // two 64-row boxes of one stored tile: rows mu of tile (I, J) at columns nu of this
+                            // K-step (K-major), or, above the diagonal, rows nu of tile (J, I) (MN-major halves)
+                            const int I = t.m0 / TM, J = ks >> 1, half = ks & 1, za = s * args.naux + t.P;
+                            const bool low = I >= J;
+                            const int y0 = low ? (I * (I + 1) / 2 + J) * TM : (J * (J + 1) / 2 + I) * TM + half * KS;
+                            tma_load_3d(dst, &mapA, low ? half * KS : 0, y0, za, &a_full[slot]);
+                            tma_load_3d(dst + A_BYTES / 2, &mapA, low ? half * KS : KS, low ? y0 + KS : y0, za, &a_full[slot]);
                         } else {
-                            const int y0 = (J * (J + 1) / 2 + I) * TM + half * KS;
-                            tma_load_3d(dst, &mapA, 0, y0, za, &a_full[slot]);
-                            tma_load_3d(dst + A_BYTES / 2, &mapA, KS, y0, za, &a_full[slot]);
+                            tma_load_3d(dst, &mapA, kx, t.m0, MODE == 1 ? s * args.nkb + kb : s, &a_full[slot]);
                         }
-                    } else {
-                        tma_load_3d(smem + slot * A_BYTES, &mapA, kx, m0, za, &a_full[slot]);
                     }
-                    ++a_issued;
-                }
-                if (!ok) break;
-            }
-            // copies in flight complete before the kernel may leave: wait (bounded) for the last ones of every
-            // slot. After a normal run the MMA issuer has consumed them all and these waits return at once;
-            // after a timeout (here or in the issuer, which may give up while this thread has finished its
-            // loop) they keep the CTA until its copies have landed.
-            for (int it = max(0, a_issued - NA); it < a_issued; ++it) {
-                const long long t0 = clock64();
-                while (!mbar_try_wait(&a_full[it % NA], (it / NA) & 1) && clock64() - t0 < WAIT_CYCLES) {
+                    a_issued = min(a_issued + 1, NA);
+                    if (++slot == NA) {
+                        slot = 0;
+                        aph ^= 1;
+                    }
                 }
             }
-            for (int k = max(0, b_issued - 2); k < b_issued; ++k) {
-                const long long t0 = clock64();
-                while (!mbar_try_wait(&b_full[k & 1], (k >> 1) & 1) && clock64() - t0 < WAIT_CYCLES) {
-                }
+        }
+        // copies in flight complete before the kernel may leave: wait (bounded) for the last ones of every
+        // slot. After a normal run the MMA issuer has consumed them all and these waits return at once;
+        // after a timeout (here or in the issuer, which may give up while this warp has finished its
+        // loop) they keep the CTA until its copies have landed. The phase of a slot's last copy: aph for the
+        // slots filled since the ring last wrapped, the one before for the others.
+        for (int i = 0; i < a_issued; ++i) {
+            const int q = (slot + NA - 1 - i) % NA;
+            const unsigned ph = q < slot ? aph : aph ^ 1;
+            const long long t0 = clock64();
+            while (!mbar_try_wait(&a_full[q], ph) && clock64() - t0 < WAIT_CYCLES) {
+            }
+        }
+        for (int i = 0; i < b_issued; ++i) {
+            const int q = (bs + 1 - i) & 1;
+            const unsigned ph = q < bs ? bph : bph ^ 1;
+            const long long t0 = clock64();
+            while (!mbar_try_wait(&b_full[q], ph) && clock64() - t0 < WAIT_CYCLES) {
             }
         }
     } else if (warp == 5) {
         // ---------------------------------- MMA issuer ----------------------------------------
-        if (lane == 0) {
-            int chunk = 0;
-            bool ok = true;
-            for (int ks = 0; ks < ksteps && ok; ++ks) {
-                const int c = chunk_of(ks);
-                if (c != chunk) {                 // new chunk: hand the finished sums to the epilogue
-                    mma_commit(acc_full);
-                    ok = mbar_wait(acc_empty, (chunk & 1), err, wait);
+        const bool leader = elect_one();
+        const uint64_t ad0 = smem_desc(smem), bd0 = smem_desc(bbuf), adm0 = smem_desc_mn(smem);
+        int slot = 0, bs = 0;
+        unsigned aph = 0, bph = 0, cph = 1;       // cph: phase of the accumulators' release (none awaited at first)
+        bool ok = true;
+        for (int b = blockIdx.x; b < total && ok; b += gridDim.x) {
+            const Tile t = decode_tile<S, N, MODE>(args, b);
+            const unsigned nw8 = (unsigned)(MODE == 1 || MODE == 2 ? N : t.nw) >> 3;   // tile width / 8
+            const unsigned bslice = nw8 * 64;                              // bytes of a B slice / 16
+            // MODE 1: position of the K-step's first 16-block in the period of ldy / 16, of which the first
+            // cols / 16 hold orbitals (at most one in the period does not)
+            const int kper = MODE == 1 ? args.ldy / 16 : 0, klive = MODE == 1 ? args.cols / 16 : 0;
+            int kpos = MODE == 1 ? (int)((long long)t.kb0 * (KS / 16) % kper) : 0;
+            int left = 0;                                                  // K-steps left in the chunk
+            for (int ks = 0; ks < t.ksteps && ok; ++ks) {
+                bool fresh = false;
+                if (left == 0) {                  // a new chunk: the epilogue has taken the last one's sums
+                    if (!(ok = mbar_wait_warp(acc_empty, cph, err, wait))) break;
                     fence_after();
-                    chunk = c;
-                    if (!ok) break;
+                    cph ^= 1;
+                    left = CSTEPS;
+                    fresh = true;
                 }
-                const int bs = ks & 1;
-                if (!mbar_wait(&b_full[bs], (ks >> 1) & 1, err, wait)) {
-                    ok = false;
-                    break;
-                }
-                fence_after();
-                const bool first_in_chunk = ks == 0 || chunk_of(ks - 1) != c;
-                unsigned char* bset = bbuf + bs * BSET;
-                const bool mn = MODE == 3 && m0 / TM < (ks >> 1);   // A read transposed from the stored tile
-                const unsigned amaj = mn ? (1u << 15) : 0u;
-                for (int s = 0; s < S; ++s) {
-                    const int it = ks * S + s, slot = it % NA;
-                    if (!mbar_wait(&a_full[slot], (it / NA) & 1, err, wait)) {
-                        ok = false;
-                        break;
-                    }
-                    fence_after();
-                    // the B slices t < S - s are consecutive N-row tiles in shared memory and their levels
-                    // s + t consecutive N-column accumulators in TMEM, so up to 256 / N of them form one
-                    // MMA of width cnt * N (one read of the A tile per MMA instead of one per slice)
+                unsigned live = 0xf;              // 16-blocks of this K-step that take products
+                if (MODE == 1 && klive != kper) {
+                    live = 0;
 #pragma unroll
                     for (int k = 0; k < KS / 16; ++k) {
-                        // K-major: +32 B per k16; MN-major: +2 atoms of 8 K-rows (2048 B) per k16
-                        const uint64_t ad = mn ? smem_desc_mn(smem + slot * A_BYTES + k * 2048)
-                                               : smem_desc(smem + slot * A_BYTES) + (uint64_t)(k * 2);
-                        for (int t = 0; t < S - s; t += MMA_SLICES) {
-                            const int cnt = min(MMA_SLICES, S - s - t);
-                            const uint64_t bd = smem_desc(bset + t * B_BYTES) + (uint64_t)(k * 2);
-                            mma_bf16(tmem + (unsigned)((s + t) * N), ad, bd, instr_desc(TM, cnt * N) | amaj,
-                                     (first_in_chunk && s == 0 && k == 0) ? 0u : 1u);
+                        live |= (kpos < klive ? 1u : 0u) << k;
+                        kpos = kpos + 1 == kper ? 0 : kpos + 1;
+                    }
+                }
+                if (!(ok = mbar_wait_warp(&b_full[bs], bph, err, wait))) break;
+                fence_after();
+                const uint64_t bdk = bd0 + (uint64_t)(bs * (BSET >> 4));
+                const bool mn = MODE == 3 && t.m0 / TM < (ks >> 1);   // A read transposed from the stored tile
+                const unsigned amaj = mn ? (1u << 15) : 0u;
+                // the products of one K-step: for A slice s the B slices q < S - s are consecutive tiles of nw rows
+                // in shared memory and their levels s + q consecutive accumulators of nw columns in TMEM, so up to
+                // 256 / N of them form one MMA (one read of the A tile per MMA instead of one per slice). The first
+                // products of a chunk (slice 0 meets every level) overwrite.
+                auto products = [&](auto all_live) {
+#pragma unroll
+                    for (int s = 0; s < S; ++s) {
+                        if (!(ok = mbar_wait_warp(&a_full[slot], aph, err, wait))) break;
+                        fence_after();
+                        const uint64_t adk = (mn ? adm0 : ad0) + (uint64_t)(slot * (A_BYTES >> 4));
+                        bool over = fresh && s == 0;
+#pragma unroll
+                        for (int k = 0; k < KS / 16; ++k) {
+                            if (!decltype(all_live)::value && !(live >> k & 1)) continue;
+                            // K-major: +32 B per k16; MN-major: +2 atoms of 8 K-rows (2048 B) per k16
+                            const uint64_t ad = adk + (mn ? (uint64_t)(k * 128) : (uint64_t)(k * 2));
+#pragma unroll
+                            for (int q = 0; q < S - s; q += MMA_SLICES) {
+                                const int cnt = MMA_SLICES < S - s - q ? MMA_SLICES : S - s - q;
+                                if (leader)
+                                    mma_bf16(tmem + (unsigned)(s + q) * nw8 * 8, ad, bdk + (uint64_t)(q * bslice + k * 2),
+                                             instr_desc(TM, 0) | (cnt * nw8) << 17 | amaj, over ? 0u : 1u);
+                            }
+                            over = false;
+                        }
+                        if (leader) mma_commit(&a_empty[slot]);
+                        if (++slot == NA) {
+                            slot = 0;
+                            aph ^= 1;
                         }
                     }
-                    mma_commit(&a_empty[slot]);
+                };
+                if (MODE != 1 || live == 0xf) products(std::true_type());
+                else products(std::false_type());
+                if (!ok) break;
+                if (leader) mma_commit(&b_empty[bs]);
+                bs ^= 1;
+                if (bs == 0) bph ^= 1;
+                --left;
+                if (left == 0 || ks + 1 == t.ksteps) {   // the chunk's sums are complete
+                    if (leader) mma_commit(acc_full);
+                    left = 0;
                 }
-                if (ok) mma_commit(&b_empty[bs]);
             }
-            if (ok && ksteps > 0) mma_commit(acc_full);
-            // every MMA this thread issued has completed before tensor memory is released
-            mma_commit(mma_done);
-            const long long t0 = clock64();
-            while (!mbar_try_wait(mma_done, 0) && clock64() - t0 < WAIT_CYCLES) {
-            }
+        }
+        // every MMA this warp issued has completed before tensor memory is released
+        if (leader) mma_commit(mma_done);
+        const long long t0 = clock64();
+        while (!mbar_try_wait(mma_done, 0) && clock64() - t0 < WAIT_CYCLES) {
         }
     } else {
         // ---------------------------------- epilogue (warps 0-3) ------------------------------
-        // MODE 0 and 2: exponents are the same for every chunk, so chunk sums are accumulated with the
+        // MODE 0, 2 and 3: exponents are the same for every chunk, so chunk sums are accumulated with the
         // level factor 2^{-7(L+2)} only and the row/column powers of two are applied once at the end.
         const int row = warp * 32 + lane;               // TMEM lane = tile row
-        const int grow = m0 + row;
-        float hi[N], lo[N];
-#pragma unroll
-        for (int c = 0; c < N; ++c) hi[c] = lo[c] = 0.f;
         const unsigned lane_base = tmem + ((unsigned)(warp * 32) << 16);
-        for (int ch = 0; ch < nchunks; ++ch) {
-            int erow = 0;
-            long long blk = 0;
-            if (MODE == 1) {
-                blk = p0 + ch;
-                erow = (grow < args.np) ? args.row_e[blk * args.np + grow] : 0;
-            }
-            if (!mbar_wait(acc_full, ch & 1, err, wait)) break;
-            fence_after();
-            // per element the levels are added in descending order; column exponents (MODE 1) are read
-            // per 16-column group to keep them out of the register file
+        constexpr int NG = N / 16;                       // 16-column groups
+        unsigned cph = 0;
+        bool ok = true;
+        for (int b = blockIdx.x; b < total && ok; b += gridDim.x) {
+            const Tile t = decode_tile<S, N, MODE>(args, b);
+            const int grow = t.m0 + row;
+            const int nw = MODE == 1 || MODE == 2 ? N : t.nw;
+            const int nchunks = (t.ksteps + CSTEPS - 1) / CSTEPS;
+            f2 hi[N / 2], lo[N / 2];
 #pragma unroll
-            for (int c0 = 0; c0 < N; c0 += 16) {
-                int ce[16];
+            for (int c = 0; c < N / 2; ++c) hi[c] = lo[c] = 0;
+            for (int ch = 0; ch < nchunks; ++ch) {
+                int erow = 0;
+                int ec[(N + 31) / 32];                   // MODE 1: column exponents, one per lane
                 if (MODE == 1) {
+                    const int* e = args.row_e + (long long)(t.chunk0 + ch) * args.np;
+                    erow = grow < args.np ? __ldg(e + grow) : 0;
 #pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        ce[j] = (n0 + c0 + j < args.np) ? __ldg(args.row_e + blk * args.np + n0 + c0 + j) : 0;
+                    for (int g = 0; g < (N + 31) / 32; ++g)
+                        ec[g] = t.n0 + g * 32 + lane < args.np ? __ldg(e + t.n0 + g * 32 + lane) : 0;
                 }
-#pragma unroll 1
-                for (int L = S - 1; L >= 0; --L) {
-                    const float lev = pow2f(-7 * (L + 2));
-                    float v[16];
-                    tmem_ld16(lane_base + (unsigned)(L * N + c0), v);
+                if (!(ok = mbar_wait_warp(acc_full, cph, err, wait))) break;
+                cph ^= 1;
+                fence_after();
+                // per element the levels are added in descending order; the next level's load is in flight while
+                // this one's sums are added
+                unsigned r[2][16];
+                tmem_ld16(lane_base + (unsigned)((S - 1) * nw), r[0]);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float sc = (MODE == 1) ? pow2f(erow + ce[j] - 7 * (L + 2)) : lev;
-                        two_sum_acc(hi[c0 + j], lo[c0 + j], v[j] * sc);
+                for (int g = 0; g < NG; ++g) {
+                    if (g * 16 < nw) {   // (a break here would keep the loop from being unrolled)
+                    // MODE 1: the factors 2^{e_row + e_col} of the group's columns; where the lowest level's
+                    // factor leaves the normal range (pow2f gives zero there) each is formed by itself
+                    f2 cf[8];
+                    int ee[16];
+                    bool plain = true;
+                    if (MODE == 1) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            ee[j] = erow + __shfl_sync(0xffffffffu, ec[g / 2], (g & 1) * 16 + j);
+                            plain = plain && ee[j] >= 7 * (S + 1) - 126 && ee[j] <= 127;
+                        }
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            cf[j] = pack2((unsigned)(127 + ee[2 * j]) << 23, (unsigned)(127 + ee[2 * j + 1]) << 23);
+                        plain = __all_sync(0xffffffffu, plain);
+                    }
+#pragma unroll
+                    for (int q = 0; q < S; ++q) {
+                        const int L = S - 1 - q, cur = (g * S + q) & 1;
+                        tmem_wait(r[cur]);
+                        if (q + 1 < S) tmem_ld16(lane_base + (unsigned)((L - 1) * nw + g * 16), r[cur ^ 1]);
+                        else if (g + 1 < NG && (g + 1) * 16 < nw)
+                            tmem_ld16(lane_base + (unsigned)((S - 1) * nw + (g + 1) * 16), r[cur ^ 1]);
+                        const unsigned lv = (unsigned)(127 - 7 * (L + 2)) << 23;
+                        const f2 lev = pack2(lv, lv);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            f2 sc = lev;
+                            if (MODE == 1) {
+                                if (plain) sc = mul2(cf[j], lev);
+                                else sc = pack2(__float_as_uint(pow2f(ee[2 * j] - 7 * (L + 2))),
+                                                __float_as_uint(pow2f(ee[2 * j + 1] - 7 * (L + 2))));
+                            }
+                            two_sum_acc(hi[g * 8 + j], lo[g * 8 + j], pack2(r[cur][2 * j], r[cur][2 * j + 1]), sc);
+                        }
+                    }
                     }
                 }
+                fence_before();
+                mbar_arrive(acc_empty);
             }
-            fence_before();
-            mbar_arrive(acc_empty);
-        }
-        // output
-        if (!*(volatile int*)err && grow < args.np) {
+            if (!ok) break;
+            // output
+            if (*(volatile int*)err || grow >= (MODE == 0 ? args.rows : args.np)) continue;
             if (MODE == 2) {
                 const int er = args.row_e[grow];
-                double* o = args.outd + (long long)grow * args.ldo + n0;
-#pragma unroll
-                for (int c = 0; c < N; ++c)
-                    o[c] = scale_pow2((double)hi[c] + (double)lo[c], er + __ldg(args.col_e + n0 + c));
-            } else if (MODE == 0 || MODE == 3) {
-                const int er = MODE == 3 ? args.row_e[P] : args.row_e[(long long)P * args.np + grow];
-                float2* o = args.out + ((long long)P * args.np + grow) * args.ldy + n0;
+                double* o = args.outd + (long long)grow * args.ldo + t.n0;
 #pragma unroll
                 for (int c = 0; c < N; ++c) {
-                    const float f = pow2f(er + __ldg(args.col_e + n0 + c));
-                    o[c] = make_float2(hi[c] * f, lo[c] * f);
+                    const f2 h = hi[c / 2], l = lo[c / 2];
+                    const double v = c & 1 ? (double)hi_of(h) + (double)hi_of(l) : (double)lo_of(h) + (double)lo_of(l);
+                    o[c] = scale_pow2(v, er + __ldg(args.col_e + t.n0 + c));
+                }
+            } else if (MODE == 0 || MODE == 3) {
+                const int er = args.row_e[MODE == 3 ? t.P : grow];
+                float2* o = args.out + ((MODE == 3 ? (long long)t.P * args.np : 0LL) + grow) * args.ldy + t.n0;
+#pragma unroll
+                for (int c = 0; c < N; ++c) {
+                    if (c < nw) {
+                        const float f = pow2f(er + __ldg(args.col_e + t.n0 + c));
+                        const f2 h = hi[c / 2], l = lo[c / 2];
+                        o[c] = c & 1 ? make_float2(hi_of(h) * f, hi_of(l) * f) : make_float2(lo_of(h) * f, lo_of(l) * f);
+                    }
                 }
             } else {
-                float2* o = args.out + ((long long)split * args.npt + grow) * args.npt + n0;
+                float2* o = args.out + ((long long)t.split * args.npt + grow) * args.npt + t.n0;
 #pragma unroll
-                for (int c = 0; c < N; ++c) o[c] = make_float2(hi[c], lo[c]);
+                for (int c = 0; c < N; c += 2)
+                    if (TM % N == 0 || t.n0 + c < args.npt) {   // a width that does not divide 128 may run over
+                        o[c] = make_float2(lo_of(hi[c / 2]), lo_of(lo[c / 2]));
+                        o[c + 1] = make_float2(hi_of(hi[c / 2]), hi_of(lo[c / 2]));
+                    }
             }
         }
     }
@@ -532,13 +692,27 @@ long long pipeline_wait_cycles() {
     return (c > 0 && c < WAIT_CYCLES) ? c : WAIT_CYCLES;
 }
 
+// CTAs that the current device holds at once: two per SM where the accumulators leave room for two (the
+// kernel's registers are bounded for it) and the rings fit twice into 228 KB
+template <int S, int N>
+int resident_ctas() {
+    int dev = 0, sms = 0;
+    DF_CUDA(cudaGetDevice(&dev));
+    DF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    return sms * (S * N <= 256 && 2 * (tc_smem_bytes<S, N>() + 1024) <= 228 * 1024 ? 2 : 1);
+}
+
 template <int S, int N, int MODE>
-void launch_tc(cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, const TcArgs& args_in, unsigned grid) {
+void launch_tc(cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& b2, const TcArgs& args_in,
+               long long total) {
+    if (total > INT_MAX - (1 << 20)) throw Error{DF_E_ARG, "tensor-core kernel: too many tiles"};
     const size_t smem = tc_smem_bytes<S, N>();
     TcArgs args = args_in;
     args.wait_cycles = pipeline_wait_cycles();
+    args.total = (int)total;
     DF_CUDA(cudaFuncSetAttribute(ozaki_tc_kernel<S, N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    ozaki_tc_kernel<S, N, MODE><<<grid, 192, smem, s>>>(a, b, args);
+    const int grid = MODE == 1 ? (int)total : (int)std::min<long long>(total, resident_ctas<S, N>());
+    ozaki_tc_kernel<S, N, MODE><<<grid, 192, smem, s>>>(a, b, b2, args);
     DF_CHECK_LAUNCH();
 }
 
@@ -568,57 +742,63 @@ void k_tc_reduce(cudaStream_t s, const float2* Kpart, int nsplit, int npt, int n
     DF_CHECK_LAUNCH();
 }
 
-// Y[P][mu][i] (float pairs) = B_P C from the slices Bs [S][naux][np][np], Cs [S][ldy][np]; CTA tiles
-// of 128 rows x N columns, N in {32, 64, 80} dividing ldy (chosen by the autotuner)
-template <int S, int N>
-void y_tc_launch(cudaStream_t s, const CUtensorMap& ma, const bf16* Cs, int np, int ldy, const TcArgs& a, int naux) {
-    const CUtensorMap mb = make_map(Cs, np, ldy, S, N);
-    const unsigned mt = (np + TM - 1) / TM;
-    launch_tc<S, N, 0>(s, ma, mb, a, (unsigned)naux * mt * (ldy / N));
+// Y[P][mu][i] (float pairs, i < cols) = B_P C from the slices of B and Cs [S][ldy][np] by tiles of 128 rows x N
+// columns (chosen by the autotuner), the last one narrower: MODE 0 from full rows, MODE 3 from packed tiles
+template <int S, int N, int MODE>
+void y_tc_launch(cudaStream_t s, const CUtensorMap& ma, const bf16* Cs, const TcArgs& a, long long row_tiles) {
+    const CUtensorMap mb = make_map(Cs, a.np, a.ldy, S, N);
+    const int last = a.cols % N;
+    const CUtensorMap mb2 = last ? make_map(Cs, a.np, a.ldy, S, (unsigned)last) : mb;
+    launch_tc<S, N, MODE>(s, ma, mb, mb2, a, row_tiles * ((a.cols + N - 1) / N));
 }
 
+// N: tile width; a tile is no wider than the columns (64 wide over 48 or fewer runs the 48-wide kernel, of which
+// two CTAs fit an SM)
+template <int MODE>
+void y_tc_dispatch(cudaStream_t s, int S, int N, const CUtensorMap& ma, const bf16* Cs, const TcArgs& a, long long row_tiles) {
+    if (N == 64 && a.cols <= 48) N = 48;
+    if (S == 3 && N == 80) y_tc_launch<3, 80, MODE>(s, ma, Cs, a, row_tiles);
+    else if (S == 5 && N == 80) y_tc_launch<5, 80, MODE>(s, ma, Cs, a, row_tiles);
+    else if (S == 3 && N == 64) y_tc_launch<3, 64, MODE>(s, ma, Cs, a, row_tiles);
+    else if (S == 5 && N == 64) y_tc_launch<5, 64, MODE>(s, ma, Cs, a, row_tiles);
+    else if (S == 3 && N == 48) y_tc_launch<3, 48, MODE>(s, ma, Cs, a, row_tiles);
+    else if (S == 5 && N == 48) y_tc_launch<5, 48, MODE>(s, ma, Cs, a, row_tiles);
+    else if (S == 3 && N == 32) y_tc_launch<3, 32, MODE>(s, ma, Cs, a, row_tiles);
+    else if (S == 5 && N == 32) y_tc_launch<5, 32, MODE>(s, ma, Cs, a, row_tiles);
+    else throw Error{DF_E_ARG, "tensor-core split Y supports 3 or 5 slices and tile widths 32, 48, 64, 80"};
+}
+
+// from full rows Bs [S][naux][np][np], exponents Be [naux][np]
 void y_split_tc(cudaStream_t s, int S, int N, const bf16* Bs, const int* Be, const bf16* Cs, const int* Ce, int naux,
-                int np, int ldy, float2* Y, int* err) {
-    if (ldy % N) throw Error{DF_E_ARG, "tensor-core split Y: tile width must divide the occupied width"};
+                int np, int ldy, int cols, float2* Y, int* err) {
+    if ((long long)naux * np > INT_MAX - TM) throw Error{DF_E_ARG, "tensor-core split Y: too many rows"};
     TcArgs a{};
-    a.mode = 0;
     a.naux = naux;
     a.np = np;
+    a.rows = naux * np;
     a.ldy = ldy;
+    a.cols = cols;
     a.row_e = Be;
     a.col_e = Ce;
     a.out = Y;
     a.err = err;
-    const CUtensorMap ma = make_map(Bs, np, np, (unsigned long long)S * naux, TM);
-    if (S == 3 && N == 80) y_tc_launch<3, 80>(s, ma, Cs, np, ldy, a, naux);
-    else if (S == 5 && N == 80) y_tc_launch<5, 80>(s, ma, Cs, np, ldy, a, naux);
-    else if (S == 3 && N == 64) y_tc_launch<3, 64>(s, ma, Cs, np, ldy, a, naux);
-    else if (S == 5 && N == 64) y_tc_launch<5, 64>(s, ma, Cs, np, ldy, a, naux);
-    else if (S == 3 && N == 32) y_tc_launch<3, 32>(s, ma, Cs, np, ldy, a, naux);
-    else if (S == 5 && N == 32) y_tc_launch<5, 32>(s, ma, Cs, np, ldy, a, naux);
-    else throw Error{DF_E_ARG, "tensor-core split Y supports 3 or 5 slices and tile widths 32, 64, 80"};
+    // the rows P np + mu as one dimension: tiles do not stop at an auxiliary row's end
+    const CUtensorMap ma = make_map(Bs, np, (unsigned long long)naux * np, S, TM);
+    y_tc_dispatch<0>(s, S, N, ma, Cs, a, ((long long)a.rows + TM - 1) / TM);
 }
 
-// Y from the packed slices Bs [S][naux][nB (nB + 1) / 2][128][128] (lower 128-tiles, one exponent Be[P]
-// per auxiliary row): tile widths as y_split_tc
-template <int S, int N>
-void y_tc_packed_launch(cudaStream_t s, const CUtensorMap& ma, const bf16* Cs, int np, int ldy, const TcArgs& a,
-                        int naux, int nB) {
-    const CUtensorMap mb = make_map(Cs, np, ldy, S, N);
-    launch_tc<S, N, 3>(s, ma, mb, a, (unsigned)naux * nB * (ldy / N));
-}
-
-// naux rows are computed; the slices of row P sit at z = s * zrows + P (zrows >= naux: the buffer's rows)
+// from the packed slices Bs [S][zrows][nB (nB + 1) / 2][128][128] (lower 128-tiles, one exponent Be[P] per
+// auxiliary row): naux rows are computed; the slices of row P sit at z = s * zrows + P (zrows >= naux: the
+// buffer's rows)
 void y_split_tc_packed(cudaStream_t s, int S, int N, const bf16* Bs, const int* Be, const bf16* Cs, const int* Ce,
-                       int naux, int zrows, int np, int nB, int ldy, float2* Y, int* err) {
-    if (ldy % N) throw Error{DF_E_ARG, "tensor-core split Y: tile width must divide the occupied width"};
+                       int naux, int zrows, int np, int nB, int ldy, int cols, float2* Y, int* err) {
     if (np > nB * TM || np % KS) throw Error{DF_E_ARG, "internal: packed tiles do not cover the padded size"};
     if (zrows < naux) throw Error{DF_E_ARG, "internal: slice buffer smaller than the rows computed"};
     TcArgs a{};
-    a.mode = 3;
     a.naux = zrows;
     a.np = np;
     a.ldy = ldy;
+    a.cols = cols;
     a.nB = nB;
     a.row_e = Be;
     a.col_e = Ce;
@@ -626,13 +806,7 @@ void y_split_tc_packed(cudaStream_t s, int S, int N, const bf16* Bs, const int* 
     a.err = err;
     const unsigned long long ntile = (unsigned long long)nB * (nB + 1) / 2;
     const CUtensorMap ma = make_map(Bs, TM, ntile * TM, (unsigned long long)S * zrows, KS);
-    if (S == 3 && N == 80) y_tc_packed_launch<3, 80>(s, ma, Cs, np, ldy, a, naux, nB);
-    else if (S == 5 && N == 80) y_tc_packed_launch<5, 80>(s, ma, Cs, np, ldy, a, naux, nB);
-    else if (S == 3 && N == 64) y_tc_packed_launch<3, 64>(s, ma, Cs, np, ldy, a, naux, nB);
-    else if (S == 5 && N == 64) y_tc_packed_launch<5, 64>(s, ma, Cs, np, ldy, a, naux, nB);
-    else if (S == 3 && N == 32) y_tc_packed_launch<3, 32>(s, ma, Cs, np, ldy, a, naux, nB);
-    else if (S == 5 && N == 32) y_tc_packed_launch<5, 32>(s, ma, Cs, np, ldy, a, naux, nB);
-    else throw Error{DF_E_ARG, "tensor-core split Y supports 3 or 5 slices and tile widths 32, 64, 80"};
+    y_tc_dispatch<3>(s, S, N, ma, Cs, a, (long long)naux * nB);
 }
 
 // B[P][c] = sum_Q L^-1[P][Q] A[Q][c] for the ncols columns of one chunk, from the 7 slices
@@ -644,7 +818,6 @@ void whiten_tc_n(cudaStream_t s, const bf16* Ls, const int* eL, const bf16* At, 
     constexpr int S = 7;
     if (kp % KS || ncols % N) throw Error{DF_E_ARG, "internal: whitening operands not padded to 64"};
     TcArgs a{};
-    a.mode = 2;
     a.naux = naux;
     a.np = naux;
     a.row_e = eL;
@@ -655,8 +828,7 @@ void whiten_tc_n(cudaStream_t s, const bf16* Ls, const int* eL, const bf16* At, 
     a.ldo = ldo;
     const CUtensorMap ma = make_map(Ls, kp, naux, S, TM);
     const CUtensorMap mb = make_map(At, kp, ncols, S, N);
-    const unsigned grid = (unsigned)((naux + TM - 1) / TM) * (unsigned)(ncols / N);
-    launch_tc<S, N, 2>(s, ma, mb, a, grid);
+    launch_tc<S, N, 2>(s, ma, mb, mb, a, (long long)((naux + TM - 1) / TM) * (ncols / N));
 }
 
 // N: output tile width, 64 or 32 (32: two CTAs per SM)
@@ -667,42 +839,41 @@ void whiten_tc(cudaStream_t s, int N, const bf16* Ls, const int* eL, const bf16*
     else throw Error{DF_E_ARG, "tensor-core whitening supports tile widths 32 and 64"};
 }
 
-// K partial sums over lower 128-tile pairs: Kpart [nsplit][npt][npt] (float pairs), from the Y slices
+// K partial sums over the lower triangle of 128-blocks: Kpart [nsplit][npt][npt] (float pairs), from the Y slices
 // Ys [S][KL / 64][np][64] (KL = naux ldy over the contraction index k = P ldy + i, tile-major) with exponents
-// Ye [chunk][np]
-template <int N>
-void k_split_tc_n(cudaStream_t s, int S, const bf16* Ys, const int* Ye, int naux, int np, int ldy, int nsplit,
-                  const int2* tiles128, int ntiles, float2* Kpart, int npt, int* err) {
+// Ye [chunk][np]. One CTA per tile: the tiles are long (hundreds of K-steps), so the block scheduler's balance is
+// worth more than a persistent CTA's overlap of their ends (measured 1341 against 1242 TFLOP/s at n = 1216).
+template <int S, int N>
+void k_tc_launch(cudaStream_t s, const bf16* Ys, TcArgs a) {
+    a.ntiles = 0;
+    for (int I = 0; I < a.npt / TM; ++I) a.ntiles += k_col_tiles(I, N);
+    const CUtensorMap ma = make_map(Ys, KS, a.np, (unsigned long long)S * a.nkb, TM);
+    const CUtensorMap mb = make_map(Ys, KS, a.np, (unsigned long long)S * a.nkb, N);
+    launch_tc<S, N, 1>(s, ma, mb, mb, a, (long long)a.ntiles * a.nsplit);
+}
+
+// N: column tile width, 32, 48 or 64
+void k_split_tc(cudaStream_t s, int S, int N, const bf16* Ys, const int* Ye, int naux, int np, int ldy, int cols, int nsplit,
+                float2* Kpart, int npt, int* err) {
     TcArgs a{};
-    a.mode = 1;
     a.naux = naux;
     a.np = np;
     a.ldy = ldy;
+    a.cols = cols;
     a.KL = (long long)naux * ldy;
     a.nkb = (int)((a.KL + KS - 1) / KS);
-    a.ntiles = ntiles;
     a.nsplit = nsplit;
     a.row_e = Ye;
-    a.tiles = tiles128;
     a.out = Kpart;
     a.npt = npt;
     a.err = err;
-    const CUtensorMap ma = make_map(Ys, KS, np, (unsigned long long)S * a.nkb, TM);
-    const CUtensorMap mb = make_map(Ys, KS, np, (unsigned long long)S * a.nkb, N);
-    const unsigned grid = (unsigned)ntiles * nsplit * (TM / N);
-    switch (S) {
-        case 3: launch_tc<3, N, 1>(s, ma, mb, a, grid); break;
-        case 5: launch_tc<5, N, 1>(s, ma, mb, a, grid); break;
-        default: throw Error{DF_E_ARG, "tensor-core split K supports 3 or 5 slices"};
-    }
-}
-
-// N: width of the column half-tiles of each 128 x 128 output tile, 64 or 32
-void k_split_tc(cudaStream_t s, int S, int N, const bf16* Ys, const int* Ye, int naux, int np, int ldy, int nsplit,
-                const int2* tiles128, int ntiles, float2* Kpart, int npt, int* err) {
-    if (N == 64) k_split_tc_n<64>(s, S, Ys, Ye, naux, np, ldy, nsplit, tiles128, ntiles, Kpart, npt, err);
-    else if (N == 32) k_split_tc_n<32>(s, S, Ys, Ye, naux, np, ldy, nsplit, tiles128, ntiles, Kpart, npt, err);
-    else throw Error{DF_E_ARG, "tensor-core split K supports tile widths 32 and 64"};
+    if (S == 3 && N == 64) k_tc_launch<3, 64>(s, Ys, a);
+    else if (S == 5 && N == 64) k_tc_launch<5, 64>(s, Ys, a);
+    else if (S == 3 && N == 48) k_tc_launch<3, 48>(s, Ys, a);
+    else if (S == 5 && N == 48) k_tc_launch<5, 48>(s, Ys, a);
+    else if (S == 3 && N == 32) k_tc_launch<3, 32>(s, Ys, a);
+    else if (S == 5 && N == 32) k_tc_launch<5, 32>(s, Ys, a);
+    else throw Error{DF_E_ARG, "tensor-core split K supports 3 or 5 slices and tile widths 32, 48, 64"};
 }
 
 }  // namespace dfhf
