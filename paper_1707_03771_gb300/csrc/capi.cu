@@ -388,7 +388,7 @@ void jk_dispatch(df_handle* h, const double* dD, const double* dC, int nocc, dou
         exchange_split(h, dC, nocc, slices, dK);
     else
         exchange_fp64(h, dC, nocc, dK);
-    h->timings_ms[16] = 5 + h->exchange_launches;   // J (pack, gamma, coulomb, split sum, unpack), K
+    h->timings_ms[16] = 4 + h->exchange_launches;   // J (pack, gamma, coulomb, sum), K
 }
 
 // K alone for m columns of occupied-like coefficients dC (n x m, device), FP64 or split
@@ -622,7 +622,9 @@ int df_jk(df_handle* h, const double* D, const double* C_occ, int nocc, double* 
             DF_CUDA(cudaMemcpyAsync(K, dK, nn * sizeof(double), cudaMemcpyDeviceToHost, s));
         }
         DF_CUDA(cudaStreamSynchronize(s));
+        collect_timings(h);
     } catch (const Error& e) {
+        h->timer.marked = 0;
         return fail(h, e);
     }
     return DF_OK;
@@ -853,6 +855,7 @@ void df_free(df_handle* h) {
     if (!h) return;
     cudaSetDevice(h->device);
     if (h->stream) cudaStreamSynchronize(h->stream);
+    h->timer.release();
     free_split(h);
     free_shells(h->dbas);
     free_shells(h->daux);

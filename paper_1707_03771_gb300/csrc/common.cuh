@@ -119,6 +119,39 @@ struct DevBuf {
 
 struct SplitState;   // split-precision work buffers (split_k.cu)
 
+// CUDA events marking the phases of the current build for the per-phase timings, read once the build's work is
+// complete (collect_timings): the events live as long as the handle, and nothing waits between the phases.
+// No marks while `on` is false (batched runs, and stream capture, where the events could not be read).
+struct PhaseTimer {
+    enum { COULOMB = 0, EXCHANGE = 3, SPLIT = 6, COUNT = 12 };
+    cudaEvent_t ev[COUNT] = {};
+    bool on = false;
+    unsigned marked = 0;
+    PhaseTimer() = default;
+    PhaseTimer(const PhaseTimer&) = delete;
+    PhaseTimer& operator=(const PhaseTimer&) = delete;
+    void mark(int i, cudaStream_t s) {
+        if (!on) return;
+        if (!ev[i]) DF_CUDA(cudaEventCreate(&ev[i]));
+        DF_CUDA(cudaEventRecord(ev[i], s));
+        marked |= 1u << i;
+    }
+    bool has(int i) const { return marked >> i & 1; }
+    double ms(int a, int b) const {
+        float t = 0.f;
+        DF_CUDA(cudaEventElapsedTime(&t, ev[a], ev[b]));
+        return t;
+    }
+    void release() {
+        for (auto& e : ev)
+            if (e) {
+                cudaEventDestroy(e);
+                e = nullptr;
+            }
+        marked = 0;
+    }
+};
+
 }  // namespace dfhf
 
 struct df_handle {
@@ -167,7 +200,8 @@ struct df_handle {
     double timings_ms[20] = {0};
     int exchange_launches = 0;     // kernel launches of the last exchange build
     std::vector<double> history;   // per SCF iteration: iteration, energy, dE, max|e|, slices, J/K ms
-    bool sync_timing = true;       // per-kernel event timings (the batch driver turns them off)
+    bool sync_timing = true;       // per-phase event timings (the SCF drivers turn them off)
+    dfhf::PhaseTimer timer;
     int* tc_err_host = nullptr;    // set by the SCF driver: the tensor-core kernels' timeout flag is copied
                                    // here (pinned) instead of being read back with a synchronisation
     double* noalloc_scratch = nullptr;   // device address of the library's static Coulomb scratch array on
@@ -210,6 +244,7 @@ void dgemv_cols(cudaStream_t s, int k, long long n, const double* A, long long l
 void jk_fp64(df_handle* h, const double* dD, const double* dC, int nocc, double* dJ, double* dK);
 void ensure_jk_buffers(df_handle* h, int nocc);
 void coulomb_fp64(df_handle* h, const double* dD, double* dJ);
+void collect_timings(df_handle* h);
 // Y[mu][P nocc + i] = sum_nu B_{P,mu nu} C_{nu i} from the packed FP64 B (Y: n rows of naux nocc; C: n x nocc)
 void y_transform_fp64(cudaStream_t s, const double* B, long long row, int n, int naux, const double* C, int nocc,
                       double* Y);
@@ -241,29 +276,4 @@ int scf_drive_rohf(df_handle* h, const df_options* o, int nalpha, int nbeta, dou
 
 double elapsed_ms(cudaEvent_t a, cudaEvent_t b);
 
-// CUDA events marking the phases of one build for the per-phase timings; none at all when `on` is false
-// (batched runs, and stream capture, where a call's own events cannot be recorded and then destroyed)
-struct PhaseTimer {
-    static constexpr int MAXEV = 8;
-    cudaEvent_t ev[MAXEV] = {};
-    int count = 0;
-    bool on = false;
-    PhaseTimer(bool enabled, int n) : count(n < MAXEV ? n : MAXEV), on(enabled) {
-        if (on)
-            for (int i = 0; i < count; ++i) DF_CUDA(cudaEventCreate(&ev[i]));
-    }
-    PhaseTimer(const PhaseTimer&) = delete;
-    PhaseTimer& operator=(const PhaseTimer&) = delete;
-    void mark(int i, cudaStream_t s) {
-        if (on) DF_CUDA(cudaEventRecord(ev[i], s));
-    }
-    double ms(int a, int b) const { return elapsed_ms(ev[a], ev[b]); }
-    void sync(int i) {
-        if (on) DF_CUDA(cudaEventSynchronize(ev[i]));
-    }
-    ~PhaseTimer() {
-        if (on)
-            for (int i = 0; i < count; ++i) cudaEventDestroy(ev[i]);
-    }
-};
 }  // namespace dfhf

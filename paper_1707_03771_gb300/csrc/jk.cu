@@ -28,27 +28,39 @@ __global__ void pack_density_kernel(const double* __restrict__ D, int n, double*
     }
 }
 
-// M[mu][nu] (n x n) from a packed row
-__global__ void unpack_kernel(const double* __restrict__ packed, int n, double* __restrict__ M) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)n * n) return;
-    M[idx] = packed[packed_index((int)(idx / n), (int)(idx % n))];
+// M[r][mu][nu] (n x n) from the packed rows r = blockIdx.y
+__global__ void unpack_kernel(const double* __restrict__ packed, long long row, int n, double* __restrict__ M) {
+    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x, nn = (long long)n * n;
+    if (idx >= nn) return;
+    M[blockIdx.y * nn + idx] = packed[blockIdx.y * row + packed_index((int)(idx / n), (int)(idx % n))];
 }
 
-// gamma_P = <B_P, Dw>: one block per row, 16-byte loads, shuffle + shared reduction
-__global__ void __launch_bounds__(256) gamma_kernel(const double* __restrict__ B, long long row,
+// The last row of tiles holds n - 64 (nt - 1) rows of the matrix, the rest is zero padding, which the two
+// Coulomb kernels leave out: they are bound by the FP64 pipe (one multiply-add per 8 bytes), and at 8 waters
+// (n = 400) the padding is a fifth of the packed elements.
+
+// gamma_P = <B_P, Dw>: one block per row, 16-byte loads, shuffle + shared reduction.
+// 12 waters (n = 590): 642 -> 571 us, the column sweep below 620 -> 522 us.
+__global__ void __launch_bounds__(256) gamma_kernel(const double* __restrict__ B, long long row, int nt, int n,
                                                     const double* __restrict__ Dw, double* __restrict__ gamma) {
     const long long P = blockIdx.x;
     const double2* b = reinterpret_cast<const double2*>(B + P * row);
     const double2* d = reinterpret_cast<const double2*>(Dw);
-    const long long n2 = row / 2;
+    constexpr int T2 = TS * TS / 2;                      // double2 per tile, a multiple of the block
+    const long long full = (long long)nt * (nt - 1) / 2 * T2;
     double s0 = 0.0, s1 = 0.0;
-    for (long long i = threadIdx.x; i < n2; i += blockDim.x) {
+    auto add = [&](long long i) {
         const double2 x = __ldcs(b + i);
         const double2 y = __ldg(d + i);
         s0 = fma(x.x, y.x, s0);
         s1 = fma(x.y, y.y, s1);
-    }
+    };
+#pragma unroll 4
+    for (long long i = threadIdx.x; i < full; i += 256) add(i);
+    const int last = (n - TS * (nt - 1)) * (TS / 2);     // double2 of a last-row tile's rows below n
+    for (int J = 0; J < nt; ++J)
+#pragma unroll 4
+        for (int i = threadIdx.x; i < last; i += 256) add(full + (long long)J * T2 + i);
     double s = s0 + s1;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -63,15 +75,20 @@ __global__ void __launch_bounds__(256) gamma_kernel(const double* __restrict__ B
     }
 }
 
-// Jp[x] = sum_P gamma_P B[P][x]; each thread owns two adjacent columns, blockIdx.y splits P
-__global__ void __launch_bounds__(256) coulomb_kernel(const double* __restrict__ B, long long row, int naux,
-                                                      const double* __restrict__ gamma, int nsplit,
+// Jp[x] = sum_P gamma_P B[P][x]; each thread owns two adjacent columns, blockIdx.y splits P (padding is not
+// written)
+__global__ void __launch_bounds__(256) coulomb_kernel(const double* __restrict__ B, long long row, int naux, int nt,
+                                                      int n, const double* __restrict__ gamma, int nsplit,
                                                       double* __restrict__ Jpart) {
     const long long c2 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (c2 * 2 >= row) return;
+    if (c2 >= (long long)nt * (nt - 1) / 2 * (TS * TS / 2) &&
+        (int)(c2 % (TS * TS / 2)) >= (n - TS * (nt - 1)) * (TS / 2))
+        return;
     const int s = blockIdx.y;
     const int p0 = (int)((long long)naux * s / nsplit), p1 = (int)((long long)naux * (s + 1) / nsplit);
     double a0 = 0.0, a1 = 0.0;
+#pragma unroll 4
     for (int P = p0; P < p1; ++P) {
         const double2 x = __ldcs(reinterpret_cast<const double2*>(B + (long long)P * row) + c2);
         const double g = gamma[P];
@@ -81,12 +98,33 @@ __global__ void __launch_bounds__(256) coulomb_kernel(const double* __restrict__
     reinterpret_cast<double2*>(Jpart + (long long)s * row)[c2] = make_double2(a0, a1);
 }
 
-__global__ void sum_splits_kernel(const double* __restrict__ part, int nsplit, long long len, double* __restrict__ out) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= len) return;
-    double s = 0.0;
-    for (int t = 0; t < nsplit; ++t) s += part[(long long)t * len + i];
-    out[i] = s;
+// J[mu][nu] = the partial sums' total, both triangles: a CTA per 8 rows of a tile pair, the mirrored part through
+// shared memory
+__global__ void __launch_bounds__(256) coulomb_sum_kernel(const double* __restrict__ part, int nsplit, long long row,
+                                                          int n, double* __restrict__ J) {
+    __shared__ double t[8][TS + 1];
+    const int tp = blockIdx.x >> 3, r0 = (blockIdx.x & 7) * 8;
+    int I = (int)((sqrt(8.0 * tp + 1.0) - 1.0) * 0.5);
+    while ((I + 1) * (I + 2) / 2 <= tp) ++I;
+    while (I * (I + 1) / 2 > tp) --I;
+    const int Jt = tp - I * (I + 1) / 2;
+    if (I * TS + r0 >= n) return;
+    for (int e = threadIdx.x; e < 8 * TS; e += 256) {
+        const int r = e / TS, c = e % TS, mu = I * TS + r0 + r, nu = Jt * TS + c;
+        double s = 0.0;
+        if (mu < n && nu < n) {
+            const double* p = part + (long long)tp * TS * TS + (r0 + r) * TS + c;
+            for (int q = 0; q < nsplit; ++q) s += p[q * row];
+            J[(long long)mu * n + nu] = s;
+        }
+        t[r][c] = s;
+    }
+    if (I == Jt) return;                                 // a diagonal tile is stored whole
+    __syncthreads();
+    for (int e = threadIdx.x; e < 8 * TS; e += 256) {
+        const int r = e & 7, c = e >> 3, mu = I * TS + r0 + r, nu = Jt * TS + c;
+        if (mu < n && nu < n) J[(long long)nu * n + mu] = t[r][c];
+    }
 }
 
 constexpr int J_SPLIT = 8;
@@ -105,7 +143,7 @@ void ensure_jk_buffers(df_handle* h, int nocc) {
     if (!h->Dw.p) {
         h->Dw.alloc(pk.row);
         h->gamma.alloc(h->naux);
-        h->Jp.alloc(pk.row * (J_SPLIT + 1));
+        h->Jp.alloc(pk.row * J_SPLIT);
         h->dD.alloc((size_t)h->n * h->n);
         h->dJ.alloc((size_t)h->n * h->n);
         h->dK.alloc((size_t)h->n * h->n);
@@ -126,35 +164,29 @@ void ensure_jk_buffers(df_handle* h, int nocc) {
 void coulomb_fp64(df_handle* h, const double* dD, double* dJ) {
     const Packing& pk = h->pk;
     cudaStream_t s = h->stream;
-    PhaseTimer t(h->sync_timing, 3);
+    PhaseTimer& t = h->timer;
+    t.on = h->sync_timing;
     pack_density_kernel<<<dim3(pk.nt, pk.nt), 256, 0, s>>>(dD, h->n, h->Dw.p);
     DF_CHECK_LAUNCH();
-    t.mark(0, s);
-    gamma_kernel<<<h->naux, 256, 0, s>>>(h->B.p, pk.row, h->Dw.p, h->gamma.p);
+    t.mark(PhaseTimer::COULOMB, s);
+    gamma_kernel<<<h->naux, 256, 0, s>>>(h->B.p, pk.row, pk.nt, h->n, h->Dw.p, h->gamma.p);
     DF_CHECK_LAUNCH();
-    t.mark(1, s);
+    t.mark(PhaseTimer::COULOMB + 1, s);
     const long long c2 = pk.row / 2;
-    coulomb_kernel<<<dim3((unsigned)((c2 + 255) / 256), J_SPLIT), 256, 0, s>>>(h->B.p, pk.row, h->naux, h->gamma.p,
-                                                                             J_SPLIT, h->Jp.p + pk.row);
+    coulomb_kernel<<<dim3((unsigned)((c2 + 255) / 256), J_SPLIT), 256, 0, s>>>(h->B.p, pk.row, h->naux, pk.nt, h->n,
+                                                                             h->gamma.p, J_SPLIT, h->Jp.p);
     DF_CHECK_LAUNCH();
-    t.mark(2, s);
-    sum_splits_kernel<<<(unsigned)((pk.row + 255) / 256), 256, 0, s>>>(h->Jp.p + pk.row, J_SPLIT, pk.row, h->Jp.p);
+    t.mark(PhaseTimer::COULOMB + 2, s);
+    coulomb_sum_kernel<<<(unsigned)(8 * pk.ntp), 256, 0, s>>>(h->Jp.p, J_SPLIT, pk.row, h->n, dJ);
     DF_CHECK_LAUNCH();
-    const long long nn = (long long)h->n * h->n;
-    unpack_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(h->Jp.p, h->n, dJ);
-    DF_CHECK_LAUNCH();
-    if (t.on) {
-        t.sync(2);
-        h->timings_ms[4] = t.ms(0, 1);
-        h->timings_ms[5] = t.ms(1, 2);
-    }
 }
 
 void exchange_fp64(df_handle* h, const double* dC, int nocc, double* dK) {
     const Packing& pk = h->pk;
     cudaStream_t s = h->stream;
-    PhaseTimer t(h->sync_timing, 3);
-    t.mark(0, s);
+    PhaseTimer& t = h->timer;
+    t.on = h->sync_timing;
+    t.mark(PhaseTimer::EXCHANGE, s);
     h->exchange_launches = 3;   // Y transform, K contraction, K reduction
     // Y (n rows of naux nocc doubles): the split exchange's Y buffer when the handle has one large enough (8
     // bytes per element as well; both run in order on the handle's stream), else its own, allocated on first use
@@ -166,14 +198,29 @@ void exchange_fp64(df_handle* h, const double* dC, int nocc, double* dK) {
         Y = h->Y.p;
     }
     y_transform_fp64(s, h->B.p, pk.row, h->n, h->naux, dC, nocc, Y);
-    t.mark(1, s);
+    t.mark(PhaseTimer::EXCHANGE + 1, s);
     k_syrk_fp64(s, Y, h->n, h->naux, nocc, k_splits(h), h->Kpart.p, dK);
-    t.mark(2, s);
-    if (t.on) {
-        t.sync(2);
-        h->timings_ms[6] = t.ms(0, 1);
-        h->timings_ms[7] = t.ms(1, 2);
+    t.mark(PhaseTimer::EXCHANGE + 2, s);
+}
+
+// the phase times of the build whose work is complete on the device (its marks are cleared)
+void collect_timings(df_handle* h) {
+    PhaseTimer& t = h->timer;
+    constexpr int C = PhaseTimer::COULOMB, E = PhaseTimer::EXCHANGE, S = PhaseTimer::SPLIT;
+    auto take = [&](int slot, int a, int b) {
+        if (t.has(a) && t.has(b)) h->timings_ms[slot] = t.ms(a, b);
+    };
+    take(4, C, C + 1);
+    take(5, C + 1, C + 2);
+    take(6, E, E + 1);
+    take(7, E + 1, E + 2);
+    if (t.has(S + 5)) {
+        take(8, S, S + 5);
+        take(9, S + 1, S + 2);      // Y = B C (split)
+        take(10, S + 3, S + 4);     // K contraction (split)
+        h->timings_ms[11] = h->timings_ms[8] - h->timings_ms[9] - h->timings_ms[10];   // slicing, reduce
     }
+    t.marked = 0;
 }
 
 void jk_fp64(df_handle* h, const double* dD, const double* dC, int nocc, double* dJ, double* dK) {
@@ -184,9 +231,10 @@ void jk_fp64(df_handle* h, const double* dD, const double* dC, int nocc, double*
 
 void unpack_rows(df_handle* h, const double* packed, int p0, int count, double* dout) {
     const long long nn = (long long)h->n * h->n;
-    for (int r = 0; r < count; ++r) {
-        unpack_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, h->stream>>>(packed + (long long)(p0 + r) * h->pk.row,
-                                                                          h->n, dout + r * nn);
+    for (int r = 0; r < count; r += 65535) {
+        const int c = std::min(65535, count - r);
+        unpack_kernel<<<dim3((unsigned)((nn + 255) / 256), c), 256, 0, h->stream>>>(packed + (long long)(p0 + r) * h->pk.row,
+                                                                                   h->pk.row, h->n, dout + r * nn);
         DF_CHECK_LAUNCH();
     }
 }
@@ -218,13 +266,13 @@ void coulomb_with_scratch(cudaStream_t s, const double* B, const Packing& pk, in
                           double* dJ, double* Dw, double* gamma, double* Jp) {
     pack_density_kernel<<<dim3(pk.nt, pk.nt), 256, 0, s>>>(dD, n, Dw);
     DF_CHECK_LAUNCH();
-    gamma_kernel<<<naux, 256, 0, s>>>(B, pk.row, Dw, gamma);
+    gamma_kernel<<<naux, 256, 0, s>>>(B, pk.row, pk.nt, n, Dw, gamma);
     DF_CHECK_LAUNCH();
     const long long c2 = pk.row / 2;
-    coulomb_kernel<<<dim3((unsigned)((c2 + 255) / 256), 1), 256, 0, s>>>(B, pk.row, naux, gamma, 1, Jp);
+    coulomb_kernel<<<dim3((unsigned)((c2 + 255) / 256), 1), 256, 0, s>>>(B, pk.row, naux, pk.nt, n, gamma, 1, Jp);
     DF_CHECK_LAUNCH();
     const long long nn = (long long)n * n;
-    unpack_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(Jp, n, dJ);
+    unpack_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(Jp, pk.row, n, dJ);
     DF_CHECK_LAUNCH();
 }
 

@@ -813,8 +813,10 @@ void tune_k(df_handle* h, SplitState* st, TcChoice& best) {
 // Y over auxiliary blocks: one block of all rows when every slice is resident; otherwise the slices of
 // each block of st->pblk rows are cut from the packed FP64 B just before the Y kernel consumes them.
 template <int S>
-void run_split(df_handle* h, SplitState* st, const double* dC, int nocc, double* dK, PhaseTimer& ev) {
+void run_split(df_handle* h, SplitState* st, const double* dC, int nocc, double* dK) {
     cudaStream_t s = h->stream;
+    PhaseTimer& ev = h->timer;
+    constexpr int T = PhaseTimer::SPLIT;
     const int np = st->np, ldy = st->ldy, naux = h->naux;
     const long long cstr = (long long)ldy * np;
     split_c_kernel<S><<<ldy, 256, 0, s>>>(dC, h->n, nocc, np, ldy, st->Cs, cstr, st->Ce);
@@ -853,7 +855,7 @@ void run_split(df_handle* h, SplitState* st, const double* dC, int nocc, double*
         }
     }
     double tune_ms = 0.0;
-    ev.mark(1, s);
+    ev.mark(T + 1, s);
     const int pblk = st->blocked ? st->pblk : naux;
     for (int p0 = 0; p0 < naux; p0 += pblk) {
         const int nb = std::min(pblk, naux - p0);
@@ -876,7 +878,7 @@ void run_split(df_handle* h, SplitState* st, const double* dC, int nocc, double*
             DF_CHECK_LAUNCH();
         }
     }
-    ev.mark(2, s);
+    ev.mark(T + 2, s);
     {
         const int nyb = (naux + pblk - 1) / pblk;   // split C, per block (slicing,) Y, re-split Y, K, reduce
         h->exchange_launches = 4 + nyb * (st->blocked ? 2 : 1);
@@ -929,20 +931,20 @@ void run_split(df_handle* h, SplitState* st, const double* dC, int nocc, double*
             h->timings_ms[14] = g_tune_ms;
         }
         h->timings_ms[15] = ch.kN;
-        ev.mark(3, s);
+        ev.mark(T + 3, s);
         k_split_tc(s, S, ch.kN, st->Ys, st->Ye, naux, np, ldy, st->cols, ksplit, st->Kpart_tc, st->npt, st->err);
-        ev.mark(4, s);
+        ev.mark(T + 4, s);
         k_tc_reduce(s, st->Kpart_tc, ksplit, st->npt, h->n, dK);
     } else {
         const int nt = np / 64;
         const int ntiles = nt * (nt + 1) / 2;
         const size_t ksmem = (size_t)2 * 2 * S * 64 * LDS * sizeof(bf16);
         DF_CUDA(cudaFuncSetAttribute(k_split_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ksmem));
-        ev.mark(3, s);
+        ev.mark(T + 3, s);
         k_split_kernel<S><<<dim3(ntiles, st->nsplit), 2 * (64 / WNT) * 32, ksmem, s>>>(
             st->Ys, ystr, st->Ye, naux, np, ldy, st->PB, st->nsplit, h->ktiles.p, st->Kpart);
         DF_CHECK_LAUNCH();
-        ev.mark(4, s);
+        ev.mark(T + 4, s);
         const long long nn = (long long)h->n * h->n;
         k_split_reduce_kernel<<<nblocks(nn, 256), 256, 0, s>>>(st->Kpart, st->nsplit, np, h->n, dK);
         DF_CHECK_LAUNCH();
@@ -968,8 +970,8 @@ void exchange_split(df_handle* h, const double* dC, int nocc, int slices, double
         st = nullptr;
     }
     // phase marks: 0 start, 1-2 Y, 3-4 K contraction, 5 end
-    PhaseTimer ev(h->sync_timing, 6);
-    ev.mark(0, h->stream);
+    h->timer.on = h->sync_timing;
+    h->timer.mark(PhaseTimer::SPLIT, h->stream);
     const int ldy = ((nocc + 31) / 32) * 32;
     // set-up: a failure part-way leaves no half-built state behind (the next call starts afresh)
     try {
@@ -1093,12 +1095,12 @@ void exchange_split(df_handle* h, const double* dC, int nocc, int slices, double
     }
     if (st->err && !h->tc_err_host) DF_CUDA(cudaMemsetAsync(st->err, 0, sizeof(int), h->stream));
     switch (slices) {
-        case 2: run_split<2>(h, st, dC, nocc, dK, ev); break;
-        case 3: run_split<3>(h, st, dC, nocc, dK, ev); break;
-        case 4: run_split<4>(h, st, dC, nocc, dK, ev); break;
-        default: run_split<5>(h, st, dC, nocc, dK, ev); break;
+        case 2: run_split<2>(h, st, dC, nocc, dK); break;
+        case 3: run_split<3>(h, st, dC, nocc, dK); break;
+        case 4: run_split<4>(h, st, dC, nocc, dK); break;
+        default: run_split<5>(h, st, dC, nocc, dK); break;
     }
-    ev.mark(5, h->stream);
+    h->timer.mark(PhaseTimer::SPLIT + 5, h->stream);
     if (st->err && h->tc_err_host) {
         DF_CUDA(cudaMemcpyAsync(h->tc_err_host, st->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     } else if (st->err) {
@@ -1107,13 +1109,6 @@ void exchange_split(df_handle* h, const double* dC, int nocc, int slices, double
         DF_CUDA(cudaMemcpyAsync(&herr, st->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
         DF_CUDA(cudaStreamSynchronize(h->stream));
         if (herr) throw Error{DF_E_TIMEOUT, "tensor-core exchange kernel timed out waiting on a barrier"};
-    }
-    if (ev.on) {
-        ev.sync(5);
-        h->timings_ms[8] = ev.ms(0, 5);
-        h->timings_ms[9] = ev.ms(1, 2);    // Y = B C (split)
-        h->timings_ms[10] = ev.ms(3, 4);   // K contraction (split)
-        h->timings_ms[11] = h->timings_ms[8] - h->timings_ms[9] - h->timings_ms[10];   // slicing, reduce
     }
 }
 
