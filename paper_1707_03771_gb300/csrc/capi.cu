@@ -16,8 +16,7 @@ namespace dfhf {
 
 void rys_eval(const double* dT, int count, int n, double* dx, double* dw, cudaStream_t s);
 const double* rys_table_host();
-void whiten_ozaki(cudaStream_t s, int naux, long long ncol, long long ld, const double* Linv, const double* A,
-                  double* B);
+void whiten_ozaki(cudaStream_t s, int naux, int n, long long ld, const double* Linv, const double* A, double* B);
 void whiten_float_float(cudaStream_t s, int m, long long ncol, const double* Linv, double* Lff, double* A, double* B,
                         long long ld, bool restore_a);
 void coulomb_kernels_load();
@@ -336,10 +335,10 @@ void build_B(df_handle* h, double tau, bool keep, int whitening) {
         lff.release();
     } else if (keep) {
         h->B.alloc(rows);
-        whiten_ozaki(s, na, h->pk.row, h->pk.row, h->Linv.p, h->A3c.p, h->B.p);
+        whiten_ozaki(s, na, h->n, h->pk.row, h->Linv.p, h->A3c.p, h->B.p);
     } else {
         // in place: the unwhitened tensor's memory becomes B
-        whiten_ozaki(s, na, h->pk.row, h->pk.row, h->Linv.p, h->A3c.p, h->A3c.p);
+        whiten_ozaki(s, na, h->n, h->pk.row, h->Linv.p, h->A3c.p, h->A3c.p);
         h->B.p = h->A3c.p;
         h->B.n = h->A3c.n;
         h->A3c.p = nullptr;

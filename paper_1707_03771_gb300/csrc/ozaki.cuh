@@ -45,26 +45,66 @@ __host__ __device__ __forceinline__ long long rint_pow2(double v, int k) {
         return (long long)rint(ldexp(ldexp(v, a), k - a));
     }
     if (d >= 54) return 0;                            // |v 2^k| < 2^53 2^-54 = 1/2
-    const long long m = (long long)((b & 0xfffffffffffffULL) | 0x10000000000000ULL);
-    long long q = m >> d;
-    const long long rem = m & ((1LL << d) - 1), half = 1LL << (d - 1);
-    q += (rem > half || (rem == half && (q & 1))) ? 1 : 0;
+    // ties to even by an addition before the shift: half less one, plus the lowest kept bit
+    const unsigned long long m = (b & 0xfffffffffffffULL) | 0x10000000000000ULL;
+    const long long q = (long long)((m + ((1ULL << (d - 1)) - 1) + ((m >> d) & 1)) >> d);
     return (b >> 63) ? -q : q;
 }
 
+// float(d) for |d| < 2^22 by an addition: int-to-float conversions run at an eighth of its rate
+__device__ __forceinline__ unsigned small_float_bits(int d) {
+    return __float_as_uint(__int_as_float(0x4B400000 + d) - 12582912.f);
+}
+
+// the two values' high halves (exact BF16 of the digits) as one word, a first
+__device__ __forceinline__ unsigned pack_bf16(unsigned a, unsigned b) { return __byte_perm(a, b, 0x7632); }
+
 // The digits come from one integer: T = rint(v 2^{7S-e}) (|T| <= 2^{7S}) peeled into balanced base-128
-// digits from the least significant end (d_S..d_2 in [-64, 63], d_1 the remaining quotient). Integer
-// arithmetic throughout.
+// digits from the least significant end (d_S..d_2 in [-64, 63], d_1 the remaining quotient), as the bits of
+// floats. Integer arithmetic throughout, 64 bits wide only while T needs it.
 template <int S>
-__device__ __forceinline__ void split_pow2(double v, int e, __nv_bfloat16* out, long long stride) {
+__device__ __forceinline__ void split_digits(double v, int e, unsigned (&f)[S]) {
     long long T = rint_pow2(v, 7 * S - e);
+    int t = 0;
 #pragma unroll
     for (int s = S - 1; s >= 1; --s) {
-        const int d = (int)((T + 64) & 127) - 64;
-        out[s * stride] = __int2bfloat16_rn(d);
-        T = (T - d) >> 7;
+        if (7 * (s + 1) + 1 > 31) {                   // T still has more than 31 bits
+            const long long u = T + 64;
+            f[s] = small_float_bits((int)(u & 127) - 64);
+            T = u >> 7;
+            t = (int)T;
+        } else {
+            if (s == S - 1) t = (int)T;
+            const int u = t + 64;
+            f[s] = small_float_bits((u & 127) - 64);
+            t = u >> 7;
+        }
     }
-    out[0] = __int2bfloat16_rn((int)T);
+    f[0] = small_float_bits(S == 1 ? (int)T : t);
+}
+
+// slices of one value, and of two values that are neighbours in every slice (out 4-byte aligned)
+template <int S>
+__device__ __forceinline__ void split_pow2(double v, int e, __nv_bfloat16* out, long long stride) {
+    unsigned f[S];
+    split_digits<S>(v, e, f);
+#pragma unroll
+    for (int s = 0; s < S; ++s) out[s * stride] = __ushort_as_bfloat16((unsigned short)(f[s] >> 16));
+}
+template <int S>
+__device__ __forceinline__ void split_pow2_pair(double a, int ea, double b, int eb, __nv_bfloat16* out, long long stride) {
+    unsigned f[S], g[S];
+    split_digits<S>(a, ea, f);
+    split_digits<S>(b, eb, g);
+#pragma unroll
+    for (int s = 0; s < S; ++s) *reinterpret_cast<unsigned*>(out + s * stride) = pack_bf16(f[s], g[s]);
+}
+
+// |v| as the bits of a non-negative double, which order as their values do (a NaN counts as zero): maxima in
+// integer arithmetic, off the FP64 pipe
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return b > 0x7ff0000000000000ull ? 0 : b;
 }
 
 }  // namespace dfhf

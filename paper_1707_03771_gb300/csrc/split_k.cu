@@ -88,32 +88,38 @@ __device__ __forceinline__ void tile_of(long long tp, int& I, int& J) {
 }
 
 // rmax[P][mu] = max_nu |B_P[mu][nu]| as the bit pattern of a non-negative double (ordered like the
-// value), gathered tile by tile: rows of tile (I, J) for mu in I, its columns for mu in J (I > J)
+// value), gathered tile by tile: rows of tile (I, J) for mu in I, its columns for mu in J (I > J). The maxima are
+// integer ones: on the FP64 pipe they, not the read of B, set the time (n = 590, naux = 1619: 2.84 -> 1.28 ms).
 __global__ void __launch_bounds__(256) row_max_tiles_kernel(const double* __restrict__ B, long long row, int np,
                                                             unsigned long long* __restrict__ rmax) {
-    __shared__ double tile[64][65];
+    __shared__ unsigned long long tile[64][65];
     const long long tp = blockIdx.x, P = blockIdx.y;
     int I, J;
     tile_of(tp, I, J);
-    const double* src = B + P * row + tp * 4096;
-    for (int i = threadIdx.x; i < 4096; i += 256) tile[i >> 6][i & 63] = fabs(src[i]);
+    const double2* src = reinterpret_cast<const double2*>(B + P * row + tp * 4096);
+#pragma unroll
+    for (int i = threadIdx.x; i < 2048; i += 256) {
+        const double2 v = __ldg(src + i);
+        tile[i >> 5][(i & 31) * 2] = abs_bits(v.x);
+        tile[i >> 5][(i & 31) * 2 + 1] = abs_bits(v.y);
+    }
     __syncthreads();
     const int k = threadIdx.x >> 2, q = threadIdx.x & 3;   // row (or column) k, quarter q
-    double mr = 0.0, mc = 0.0;
+    unsigned long long mr = 0, mc = 0;
 #pragma unroll 4
     for (int j = q * 16; j < q * 16 + 16; ++j) {
-        mr = fmax(mr, tile[k][j]);
-        mc = fmax(mc, tile[j][k]);
+        mr = max(mr, tile[k][j]);
+        mc = max(mc, tile[j][k]);
     }
 #pragma unroll
     for (int o = 1; o < 4; o <<= 1) {
-        mr = fmax(mr, __shfl_xor_sync(0xffffffffu, mr, o));
-        mc = fmax(mc, __shfl_xor_sync(0xffffffffu, mc, o));
+        mr = max(mr, __shfl_xor_sync(0xffffffffu, mr, o));
+        mc = max(mc, __shfl_xor_sync(0xffffffffu, mc, o));
     }
     if (q == 0) {
         unsigned long long* rm = rmax + P * np;
-        atomicMax(rm + I * 64 + k, (unsigned long long)__double_as_longlong(mr));
-        if (I != J) atomicMax(rm + J * 64 + k, (unsigned long long)__double_as_longlong(mc));
+        atomicMax(rm + I * 64 + k, mr);
+        if (I != J) atomicMax(rm + J * 64 + k, mc);
     }
 }
 
@@ -127,8 +133,21 @@ __global__ void row_exponent_kernel(const unsigned long long* __restrict__ rmax,
     Be[i] = e;
 }
 
+// one 64 x 64 tile into shared memory
+__device__ __forceinline__ void load_tile(const double* src, double (&tile)[64][65]) {
+    const double2* s2 = reinterpret_cast<const double2*>(src);
+#pragma unroll
+    for (int i = threadIdx.x; i < 2048; i += 256) {
+        const double2 v = __ldg(s2 + i);
+        tile[i >> 5][(i & 31) * 2] = v.x;
+        tile[i >> 5][(i & 31) * 2 + 1] = v.y;
+    }
+}
+
 // slices of rows [0, nrows) of B (pointer at the block's first row): each packed tile (I, J) is read
-// once and written as block (I, J) and, for I > J, transposed as block (J, I); Be holds the block's rows
+// once and written as block (I, J) and, for I > J, transposed as block (J, I); Be holds the block's rows. A warp
+// writes 64 neighbours of a slice, two a lane. Bound by HBM with the digit arithmetic close behind (n = 590,
+// naux = 1619: 2.85 -> 1.94 ms for 3.0 GB in and 6.6 GB out).
 template <int S>
 __global__ void __launch_bounds__(256) split_b_tiles_kernel(const double* __restrict__ B, long long row, int np,
                                                             const int* __restrict__ Be, bf16* __restrict__ Bs,
@@ -137,21 +156,19 @@ __global__ void __launch_bounds__(256) split_b_tiles_kernel(const double* __rest
     const long long tp = blockIdx.x, P = blockIdx.y;
     int I, J;
     tile_of(tp, I, J);
-    const double* src = B + P * row + tp * 4096;
-    for (int i = threadIdx.x; i < 4096; i += 256) tile[i >> 6][i & 63] = src[i];
+    load_tile(B + P * row + tp * 4096, tile);
     __syncthreads();
     const int* e = Be + P * np;
     bf16* out = Bs + P * np * (long long)np;
-    for (int i = threadIdx.x; i < 4096; i += 256) {   // block (I, J): mu = I*64 + r, nu = J*64 + c
-        const int r = i >> 6, c = i & 63;
-        const int mu = I * 64 + r;
-        split_pow2<S>(tile[r][c], e[mu], out + (long long)mu * np + J * 64 + c, sstride);
+    const int c = (threadIdx.x & 31) * 2;
+    for (int r = threadIdx.x >> 5; r < 64; r += 8) {   // block (I, J): mu = I*64 + r, nu = J*64 + c
+        const int mu = I * 64 + r, em = __ldg(e + mu);
+        split_pow2_pair<S>(tile[r][c], em, tile[r][c + 1], em, out + (long long)mu * np + J * 64 + c, sstride);
     }
     if (I != J)
-        for (int i = threadIdx.x; i < 4096; i += 256) {   // block (J, I): mu = J*64 + c, nu = I*64 + r
-            const int r = i & 63, c = i >> 6;
-            const int mu = J * 64 + c;
-            split_pow2<S>(tile[r][c], e[mu], out + (long long)mu * np + I * 64 + r, sstride);
+        for (int r = threadIdx.x >> 5; r < 64; r += 8) {   // block (J, I): mu = J*64 + r, nu = I*64 + c
+            const int mu = J * 64 + r, em = __ldg(e + mu);
+            split_pow2_pair<S>(tile[c][r], em, tile[c + 1][r], em, out + (long long)mu * np + I * 64 + c, sstride);
         }
 }
 
@@ -159,12 +176,16 @@ __global__ void __launch_bounds__(256) split_b_tiles_kernel(const double* __rest
 __global__ void __launch_bounds__(256) p_max_tiles_kernel(const double* __restrict__ B, long long row,
                                                           unsigned long long* __restrict__ pmax) {
     const long long tp = blockIdx.x, P = blockIdx.y;
-    const double* src = B + P * row + tp * 4096;
-    double m = 0.0;
-    for (int i = threadIdx.x; i < 4096; i += 256) m = fmax(m, fabs(src[i]));
+    const double2* src = reinterpret_cast<const double2*>(B + P * row + tp * 4096);
+    unsigned long long m = 0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(pmax + P, (unsigned long long)__double_as_longlong(m));
+    for (int i = threadIdx.x; i < 2048; i += 256) {
+        const double2 v = __ldg(src + i);
+        m = max(m, max(abs_bits(v.x), abs_bits(v.y)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(pmax + P, m);
 }
 
 // slices of rows [0, nrows) of B into the packed layout Bs[s][P][t][128][128] (lower 128-tiles
@@ -180,22 +201,18 @@ __global__ void __launch_bounds__(256) split_b_packed_kernel(const double* __res
     const long long tp = blockIdx.x, P = blockIdx.y;
     int I, J;
     tile_of(tp, I, J);
-    const double* src = B + P * row + tp * 4096;
-    for (int i = threadIdx.x; i < 4096; i += 256) tile[i >> 6][i & 63] = src[i];
+    load_tile(B + P * row + tp * 4096, tile);
     __syncthreads();
     const int e = Be[P];
     const int IB = I >> 1, JB = J >> 1;
     bf16* out = Bs + (P * ntile + (long long)IB * (IB + 1) / 2 + JB) * 16384;
     const int ro = (I & 1) * 64, co = (J & 1) * 64;
-    for (int i = threadIdx.x; i < 4096; i += 256) {
-        const int r = i >> 6, c = i & 63;
-        split_pow2<S>(tile[r][c], e, out + (ro + r) * 128 + co + c, sstride);
-    }
+    const int c = (threadIdx.x & 31) * 2;
+    for (int r = threadIdx.x >> 5; r < 64; r += 8)
+        split_pow2_pair<S>(tile[r][c], e, tile[r][c + 1], e, out + (ro + r) * 128 + co + c, sstride);
     if (IB == JB && I != J)
-        for (int i = threadIdx.x; i < 4096; i += 256) {
-            const int r = i & 63, c = i >> 6;
-            split_pow2<S>(tile[r][c], e, out + (co + c) * 128 + ro + r, sstride);
-        }
+        for (int r = threadIdx.x >> 5; r < 64; r += 8)
+            split_pow2_pair<S>(tile[c][r], e, tile[c + 1][r], e, out + (co + r) * 128 + ro + c, sstride);
 }
 
 // C (n x nocc row-major) -> Cs[s][i][nu] (ldy x np), exponent per column i

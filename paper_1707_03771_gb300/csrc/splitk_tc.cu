@@ -236,9 +236,11 @@ struct TcArgs {
     float2* out;             // MODE 0: Y [naux][np][ldy]; MODE 1: Kpart [nsplit][npt][npt]
     int npt;                 // MODE 1: padded dimension of Kpart (multiple of 128)
     int* err;
-    // MODE 2 (whitening): rows = naux (np is set to naux), ncols pair columns of this chunk,
-    // row_e = L^-1 row exponents, col_e = column exponents, output FP64 rows of stride ldo
+    // MODE 2 (whitening): rows = naux (np is set to naux), ncols pair columns of this chunk, row_e = L^-1 row
+    // exponents, col_e = column exponents, output FP64 rows of stride ldo: a column's elements go to its
+    // positions pos (its own, its mirror's; negative: none) of the row
     int ncols;
+    const int2* pos;
     double* outd;
     long long ldo;
     long long wait_cycles;   // budget of the pipeline waits (WAIT_CYCLES by default)
@@ -607,12 +609,15 @@ __global__ void __launch_bounds__(192, S * N <= 256 ? 2 : 1)
             if (*(volatile int*)err || grow >= (MODE == 0 ? args.rows : args.np)) continue;
             if (MODE == 2) {
                 const int er = args.row_e[grow];
-                double* o = args.outd + (long long)grow * args.ldo + t.n0;
+                double* o = args.outd + (long long)grow * args.ldo;
 #pragma unroll
                 for (int c = 0; c < N; ++c) {
                     const f2 h = hi[c / 2], l = lo[c / 2];
-                    const double v = c & 1 ? (double)hi_of(h) + (double)hi_of(l) : (double)lo_of(h) + (double)lo_of(l);
-                    o[c] = scale_pow2(v, er + __ldg(args.col_e + t.n0 + c));
+                    const double v = scale_pow2(c & 1 ? (double)hi_of(h) + (double)hi_of(l) : (double)lo_of(h) + (double)lo_of(l),
+                                                er + __ldg(args.col_e + t.n0 + c));
+                    const int2 p = __ldg(args.pos + t.n0 + c);
+                    if (p.x >= 0) o[p.x] = v;
+                    if (p.y >= 0) o[p.y] = v;
                 }
             } else if (MODE == 0 || MODE == 3) {
                 const int er = args.row_e[MODE == 3 ? t.P : grow];
@@ -821,12 +826,12 @@ void y_split_tc_packed(cudaStream_t s, int S, int N, const bf16* Bs, const int* 
     y_tc_dispatch<3>(s, S, N, ma, Cs, a, (long long)naux * nB);
 }
 
-// B[P][c] = sum_Q L^-1[P][Q] A[Q][c] for the ncols columns of one chunk, from the 7 slices
+// B[P][pos[c]] = sum_Q L^-1[P][Q] A[Q][c] for the ncols columns of one chunk, from the 7 slices
 // Ls [7][naux][kp] (row exponents eL) and At [7][ncols][kp] (column exponents eA); rows of `out` have
 // stride ldo. kp is naux padded to a multiple of 64 (zero slices beyond naux), ncols a multiple of 64.
 template <int N>
 void whiten_tc_n(cudaStream_t s, const bf16* Ls, const int* eL, const bf16* At, const int* eA, int naux, int kp,
-                 int ncols, double* out, long long ldo, int* err) {
+                 int ncols, const int2* pos, double* out, long long ldo, int* err) {
     constexpr int S = 7;
     if (kp % KS || ncols % N) throw Error{DF_E_ARG, "internal: whitening operands not padded to 64"};
     TcArgs a{};
@@ -836,6 +841,7 @@ void whiten_tc_n(cudaStream_t s, const bf16* Ls, const int* eL, const bf16* At, 
     a.col_e = eA;
     a.err = err;
     a.ncols = ncols;
+    a.pos = pos;
     a.outd = out;
     a.ldo = ldo;
     const CUtensorMap ma = make_map(Ls, kp, naux, S, TM);
@@ -845,9 +851,9 @@ void whiten_tc_n(cudaStream_t s, const bf16* Ls, const int* eL, const bf16* At, 
 
 // N: output tile width, 64 or 32 (32: two CTAs per SM)
 void whiten_tc(cudaStream_t s, int N, const bf16* Ls, const int* eL, const bf16* At, const int* eA, int naux, int kp,
-               int ncols, double* out, long long ldo, int* err) {
-    if (N == 64) whiten_tc_n<64>(s, Ls, eL, At, eA, naux, kp, ncols, out, ldo, err);
-    else if (N == 32) whiten_tc_n<32>(s, Ls, eL, At, eA, naux, kp, ncols, out, ldo, err);
+               int ncols, const int2* pos, double* out, long long ldo, int* err) {
+    if (N == 64) whiten_tc_n<64>(s, Ls, eL, At, eA, naux, kp, ncols, pos, out, ldo, err);
+    else if (N == 32) whiten_tc_n<32>(s, Ls, eL, At, eA, naux, kp, ncols, pos, out, ldo, err);
     else throw Error{DF_E_ARG, "tensor-core whitening supports tile widths 32 and 64"};
 }
 

@@ -9,8 +9,10 @@
 // differs from an FP64 product L^-1 A by ~3e-10 of max|B| on the 8-water cluster, well inside the
 // ~kappa(L) eps |B| by which two correct FP64 whitenings differ (8e-9 there).
 //
-// The pair columns are processed in chunks whose transposed slices fit a bounded buffer; when the
-// unwhitened tensor is not kept, each chunk's result overwrites the chunk's own columns in place.
+// The columns are the distinct pairs mu >= nu of the packed rows: the padding of the last tiles (zero) and the
+// mirror halves of the diagonal tiles (written beside their originals) are not whitened; at n = 590 they are a
+// quarter of the packed elements. The columns are processed in chunks whose transposed slices fit a bounded
+// buffer; when the unwhitened tensor is not kept, each chunk's result overwrites the chunk's own columns in place.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -24,7 +26,7 @@
 namespace dfhf {
 
 void whiten_tc(cudaStream_t s, int N, const __nv_bfloat16* Ls, const int* eL, const __nv_bfloat16* At, const int* eA,
-               int naux, int kp, int ncols, double* out, long long ldo, int* err);
+               int naux, int kp, int ncols, const int2* pos, double* out, long long ldo, int* err);
 
 namespace {
 
@@ -58,73 +60,107 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(const double* __restric
     for (int q = threadIdx.x; q < kp; q += blockDim.x) split_pow2<WS>(q < naux ? row[q] : 0.0, e, o + q, sstr);
 }
 
-// eA[c] = exponent of max_Q |A[Q][c0 + c]| for the chunk's columns
-__global__ void __launch_bounds__(256) col_exponent_kernel(const double* __restrict__ A, long long ld, int naux,
-                                                           long long c0, int nc, int* __restrict__ eA) {
+// positions of column c (the pair mu >= nu) in a packed row: its own and its mirror's in a diagonal tile (-1: none);
+// columns beyond the last pair have none
+__global__ void __launch_bounds__(256) column_positions_kernel(long long npair, long long count, int2* __restrict__ pos) {
+    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= count) return;
+    int2 p = make_int2(-1, -1);
+    if (c < npair) {
+        int mu = (int)((sqrt(8.0 * (double)c + 1.0) - 1.0) * 0.5);
+        while ((long long)(mu + 1) * (mu + 2) / 2 <= c) ++mu;
+        while ((long long)mu * (mu + 1) / 2 > c) --mu;
+        const int nu = (int)(c - (long long)mu * (mu + 1) / 2);
+        p.x = (int)packed_index(mu, nu);
+        if (mu / TS == nu / TS && mu != nu) p.y = (int)packed_index(nu, mu);
+    }
+    pos[c] = p;
+}
+
+// cmax[c] = max_Q |A[Q][column c]| as the bits of a non-negative double, over the rows of blockIdx.y; pos at the
+// chunk's first column
+__global__ void __launch_bounds__(256) col_max_kernel(const double* __restrict__ A, long long ld, int naux,
+                                                      const int2* __restrict__ pos, int nc,
+                                                      unsigned long long* __restrict__ cmax) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= nc) return;
-    const double* a = A + c0 + c;
-    double m0 = 0.0, m1 = 0.0, m2 = 0.0, m3 = 0.0;
-    int q = 0;
-    for (; q + 4 <= naux; q += 4) {
-        m0 = fmax(m0, fabs(a[(long long)q * ld]));
-        m1 = fmax(m1, fabs(a[(long long)(q + 1) * ld]));
-        m2 = fmax(m2, fabs(a[(long long)(q + 2) * ld]));
-        m3 = fmax(m3, fabs(a[(long long)(q + 3) * ld]));
-    }
-    for (; q < naux; ++q) m0 = fmax(m0, fabs(a[(long long)q * ld]));
-    const double mx = fmax(fmax(m0, m1), fmax(m2, m3));
+    const int p = pos[c].x;
+    if (p < 0) return;
+    const int q0 = (int)((long long)naux * blockIdx.y / gridDim.y), q1 = (int)((long long)naux * (blockIdx.y + 1) / gridDim.y);
+    unsigned long long m = 0;
+#pragma unroll 8
+    for (int q = q0; q < q1; ++q) m = max(m, abs_bits(A[(long long)q * ld + p]));
+    atomicMax(cmax + c, m);
+}
+
+// eA[c] = e with max 2^-e < 1 (0 for a zero column)
+__global__ void col_exponent_kernel(const unsigned long long* __restrict__ cmax, int nc, int* __restrict__ eA) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= nc) return;
+    const double mx = __longlong_as_double((long long)cmax[c]);
     int e = 0;
     if (mx > 0.0) frexp(mx, &e);
     eA[c] = e;
 }
 
-// At[s][c][Q] (kp per column, zero beyond naux) = slices of A[Q][c0 + c] 2^-eA[c]; 64 x 64 tiles
-// transposed through shared memory (reads coalesced along c, writes along Q)
+// At[s][c][Q] (kp per column, zero beyond naux) = slices of column c 2^-eA[c]; 64 x 64 tiles transposed through
+// shared memory (reads run along the packed row, a warp writes 64 neighbours along Q). n = 590, naux = 1619:
+// 2.10 -> 1.39 ms
 __global__ void __launch_bounds__(256) slice_cols_kernel(const double* __restrict__ A, long long ld, int naux, int kp,
-                                                         long long c0, const int* __restrict__ eA,
+                                                         const int2* __restrict__ pos, const int* __restrict__ eA,
                                                          bf16* __restrict__ At, long long sstr) {
     __shared__ double tile[64][65];
     const int cb = blockIdx.x * 64, q0 = blockIdx.y * 64;
     const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;   // 64 x 4
+    const int p = pos[cb + tx].x;
+#pragma unroll 4
     for (int r = ty; r < 64; r += 4) {
         const int q = q0 + r;
-        tile[r][tx] = q < naux ? A[(long long)q * ld + c0 + cb + tx] : 0.0;
+        tile[r][tx] = (q < naux && p >= 0) ? A[(long long)q * ld + p] : 0.0;
     }
     __syncthreads();
-    for (int r = ty; r < 64; r += 4) {   // r: column within the tile, tx: Q within the tile
-        const int c = cb + r;
-        split_pow2<WS>(tile[tx][r], eA[c], At + (long long)c * kp + q0 + tx, sstr);
+    const int k = (threadIdx.x & 31) * 2;
+    for (int r = threadIdx.x >> 5; r < 64; r += 8) {          // r: column within the tile, k: Q within the tile
+        const int c = cb + r, e = __ldg(eA + c);
+        split_pow2_pair<WS>(tile[k][r], e, tile[k + 1][r], e, At + (long long)c * kp + q0 + k, sstr);
     }
 }
 
 }  // namespace
 
-// B = L^-1 A for the packed tensor A (naux rows of `ncol` doubles, stride ld). `B` may equal `A`
-// (in place, chunk by chunk). Scratch: the slices of L^-1 and one chunk of transposed slices.
-void whiten_ozaki(cudaStream_t s, int naux, long long ncol, long long ld, const double* Linv, const double* A,
-                  double* B) {
-    if (ncol % 64) throw Error{DF_E_ARG, "internal: whitening columns not a multiple of 64"};
+// B = L^-1 A for the packed tensor A of n orbital functions (naux rows of stride ld). `B` may equal `A` (in place,
+// chunk by chunk); else its padding is A's. Scratch: the slices of L^-1 and one chunk of transposed slices.
+void whiten_ozaki(cudaStream_t s, int naux, int n, long long ld, const double* Linv, const double* A, double* B) {
+    if (ld > 0x7fffffff) throw Error{DF_E_ARG, "whitening supports packed rows of at most 2^31 elements"};
+    const long long npair = (long long)n * (n + 1) / 2;
+    const long long ncol = (npair + 63) / 64 * 64;
+    if (B != A) DF_CUDA(cudaMemsetAsync(B, 0, sizeof(double) * (size_t)naux * ld, s));
     const int kp = (naux + 63) / 64 * 64;
     size_t free_b = 0, total_b = 0;
     DF_CUDA(cudaMemGetInfo(&free_b, &total_b));
     const double col_bytes = (double)WS * kp * 2 + 4;
     // the chunk's transposed slices: at most 8 GB (several molecules may whiten at once)
     const double chunk_bytes = std::min(0.4 * (double)free_b, 8.0e9);
-    long long nc = (long long)std::min<double>((double)ncol, chunk_bytes / col_bytes);
-    nc = std::min<long long>(nc, 1LL << 19) / 4096 * 4096;
-    if (nc < 64) nc = std::min<long long>(ncol, 64);
-    if (nc > ncol) nc = ncol;
+    // columns per chunk: at most 2^19 and what the buffer holds, in chunks of nearly equal size
+    const long long most = std::max<long long>(64, (long long)std::min<double>(1LL << 19, chunk_bytes / col_bytes) / 64 * 64);
+    const long long chunks = (ncol + most - 1) / most;
+    const long long nc = ((ncol + chunks - 1) / chunks + 63) / 64 * 64;
     DevBuf<bf16> Ls, At;
     DevBuf<int> eL, eA, err;
+    DevBuf<int2> pos;
+    DevBuf<unsigned long long> cmax;
     Ls.alloc((size_t)WS * naux * kp);
     eL.alloc(naux);
     At.alloc((size_t)WS * nc * kp);
     eA.alloc(nc);
+    pos.alloc(ncol);
+    cmax.alloc(nc);
     err.alloc(1);
     err.zero(s);
     try {
     slice_rows_kernel<<<naux, 256, 0, s>>>(Linv, naux, kp, Ls.p, (long long)naux * kp, eL.p);
+    DF_CHECK_LAUNCH();
+    column_positions_kernel<<<(unsigned)((ncol + 255) / 256), 256, 0, s>>>(npair, ncol, pos.p);
     DF_CHECK_LAUNCH();
     const int bucket = (naux + 511) / 512;
     int tile = 0;
@@ -137,23 +173,28 @@ void whiten_ozaki(cudaStream_t s, int naux, long long ncol, long long ld, const 
         const int t = std::atoi(f);
         if (t == 32 || t == 64) tile = t;
     }
-    const bool tune = tile == 0 && ncol >= 2 * nc;   // two full-width chunks to compare
+    const bool tune = tile == 0 && chunks >= 3;      // two chunks of the same size to compare
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
     if (tune)
         for (auto& e : ev) DF_CUDA(cudaEventCreate(&e));
     int k = 0;
     for (long long c0 = 0; c0 < ncol; c0 += nc, ++k) {
         const int w = (int)std::min<long long>(nc, ncol - c0);
-        col_exponent_kernel<<<(w + 255) / 256, 256, 0, s>>>(A, ld, naux, c0, w, eA.p);
+        cmax.zero(s);
+        // enough row ranges to fill the GPU
+        const int ranges = std::max(1, std::min(naux / 16, (16 * 152 * 256 + w - 1) / w));
+        col_max_kernel<<<dim3((w + 255) / 256, ranges), 256, 0, s>>>(A, ld, naux, pos.p + c0, w, cmax.p);
         DF_CHECK_LAUNCH();
-        slice_cols_kernel<<<dim3(w / 64, kp / 64), 256, 0, s>>>(A, ld, naux, kp, c0, eA.p, At.p, (long long)w * kp);
+        col_exponent_kernel<<<(w + 255) / 256, 256, 0, s>>>(cmax.p, w, eA.p);
+        DF_CHECK_LAUNCH();
+        slice_cols_kernel<<<dim3(w / 64, kp / 64), 256, 0, s>>>(A, ld, naux, kp, pos.p + c0, eA.p, At.p, (long long)w * kp);
         DF_CHECK_LAUNCH();
         int use = tile ? tile : 64;
         if (tune && k < 2) {
             use = k == 0 ? 64 : 32;
             DF_CUDA(cudaEventRecord(ev[2 * k], s));
         }
-        whiten_tc(s, use, Ls.p, eL.p, At.p, eA.p, naux, kp, w, B + c0, ld, err.p);
+        whiten_tc(s, use, Ls.p, eL.p, At.p, eA.p, naux, kp, w, pos.p + c0, B, ld, err.p);
         if (tune && k < 2) DF_CUDA(cudaEventRecord(ev[2 * k + 1], s));
         if (tune && k == 1) {
             DF_CUDA(cudaEventSynchronize(ev[3]));
