@@ -240,6 +240,11 @@ void dgemm_lower(cudaStream_t s, int m, int n, int k, double alpha, const double
 void dgemv_rows(cudaStream_t s, int m, long long k, const double* A, long long lda, const double* x, double* y);
 void dgemv_cols(cudaStream_t s, int k, long long n, const double* A, long long lda, const double* x, double* y);
 
+// small symmetric eigenproblems (jacobi.cu)
+constexpr int JACOBI_MAX = 160;
+size_t jacobi_work_doubles(int n);
+void jacobi_eig(cudaStream_t s, int n, const double* A, double* w, double* out, double* work, int* info);
+
 // J/K (jk.cu)
 void jk_fp64(df_handle* h, const double* dD, const double* dC, int nocc, double* dJ, double* dK);
 void ensure_jk_buffers(df_handle* h, int nocc);

@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "grid_barrier.cuh"
 
 struct df_mlp {
     int nin = 0, nh = 0, nlayers = 0, nout = 0;   // nlayers hidden layers of width nh
@@ -56,7 +57,6 @@ constexpr int stage_k() {
 constexpr int UO = 4;               // outputs of a weight-update task
 constexpr int UR = 64;              // rows of a weight-update task staged at once
 constexpr int MAX_SHARED_LAYERS = 32;
-constexpr long long GRID_WAIT_CYCLES = 4000000000LL;   // about 2 s
 
 struct Layer {
     int ni, no;
@@ -78,32 +78,6 @@ struct StepArgs {
     unsigned* count;                // barrier arrivals
     int* err;
 };
-
-// all CTAs of the grid (co-resident: a cooperative launch); false on every thread if the wait expires
-__device__ bool grid_barrier(unsigned* count, int* err, unsigned& target) {
-    __shared__ int ok;
-    __syncthreads();
-    target += gridDim.x;
-    if (threadIdx.x == 0) {
-        int good = 1;
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(count) : "memory");
-        const long long t0 = clock64();
-        // arrivals only grow; the difference is taken modulo 2^32
-        for (;;) {
-            unsigned seen;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(seen) : "l"(count) : "memory");
-            if ((int)(seen - target) >= 0) break;
-            if (clock64() - t0 > GRID_WAIT_CYCLES || *(volatile int*)err) {
-                atomicExch(err, DF_E_TIMEOUT);
-                good = 0;
-                break;
-            }
-        }
-        ok = good;
-    }
-    __syncthreads();
-    return ok != 0;
-}
 
 // kz floats of a row into shared memory (those from kc on, or all of a missing row, as zeros), by one warp: 16
 // bytes a lane where source and count allow it, else 4

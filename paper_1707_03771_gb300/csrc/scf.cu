@@ -8,7 +8,8 @@
 // e = 2 (F' P - P F') with P = V_occ V_occ^T, the extrapolation combines the F' of earlier iterations,
 // and only the occupied orbitals C_occ = X V_occ are formed each iteration.
 // Every step runs on the device in FP64 (DIIS included); only the energy and max|e| cross to the
-// host each iteration for the convergence test. The symmetric eigensolver is cuSOLVER's dsyevd.
+// host each iteration for the convergence test. The symmetric eigensolver is cuSOLVER's dsyevd, for the small
+// matrices of FP64 runs jacobi.cu's.
 #include <algorithm>
 #include <chrono>
 #include <cstdio>
@@ -816,12 +817,44 @@ class ScfRun {
         }
     }
 
+    // the eigensolver of the FP64 runs' small matrices is jacobi.cu's. Split-precision runs (and the atoms of the
+    // SAD guess that starts them) keep cuSOLVER's at every size: their early 3-slice exchange depends on the last
+    // bits of the orbitals, so another solver's rotations within the occupied space would show in their results.
+    bool own_eig(int m) const { return o_.precision == DF_PREC_FP64 && !frac_ && m <= JACOBI_MAX; }
+
     void eig(double* A, int m, double* w) {
+        if (own_eig(m)) {
+            if (m > jac_n_) {
+                if (jac_) cudaFree(jac_);
+                jac_ = nullptr;
+                jac_n_ = std::min(JACOBI_MAX, std::max(m, n_));
+                DF_CUDA(cudaMalloc((void**)&jac_, sizeof(double) * jacobi_work_doubles(jac_n_)));
+            }
+            jacobi_eig(s_, m, A, w, A, jac_, info_);
+            return;
+        }
         int lw = 0;
         DF_SOLVER(cusolverDnDsyevd_bufferSize(h_->solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_UPPER, m, A, m, w, &lw));
         grow_work(lw);
         DF_SOLVER(cusolverDnDsyevd(h_->solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_UPPER, m, A, m, w, work_,
                                    lwork_, info_));
+    }
+
+    // eigenvectors of the Fock matrix in Fp_ (in place) in the basis of the last iteration's (vlast_), where it is
+    // nearly diagonal late in the SCF and Jacobi needs few sweeps: A = V F V^T, V <- V_A V. One basis per run.
+    void eig_from_last() {
+        const long long no = (long long)nX_ * nX_;
+        if (!vlast_) {
+            DF_CUDA(cudaMalloc((void**)&vlast_, sizeof(double) * 2 * no));
+            eig(Fp_, nX_, h_->eps.p);
+        } else {
+            double* T = vlast_ + no;
+            mm(s_, false, false, nX_, nX_, nX_, 1.0, vlast_, nX_, Fp_, nX_, 0.0, T, nX_);
+            mm(s_, false, true, nX_, nX_, nX_, 1.0, T, nX_, vlast_, nX_, 0.0, Fp_, nX_);
+            jacobi_eig(s_, nX_, Fp_, h_->eps.p, T, jac_, info_);
+            mm(s_, false, false, nX_, nX_, nX_, 1.0, T, nX_, vlast_, nX_, 0.0, Fp_, nX_);
+        }
+        DF_CUDA(cudaMemcpyAsync(vlast_, Fp_, sizeof(double) * no, cudaMemcpyDeviceToDevice, s_));
     }
 
     // Fo = X^T Fm X (nX x nX)
@@ -874,7 +907,8 @@ class ScfRun {
             return;
         }
         mixed_step_ = false;
-        eig(Fp_, nX_, h_->eps.p);
+        if (own_eig(nX_)) eig_from_last();
+        else eig(Fp_, nX_, h_->eps.p);
         vt_ = Fp_;
         fock_basis_ = true;
         if (frac_) weight_occupied();
@@ -1002,6 +1036,10 @@ class ScfRun {
         f32lwork_ = 0;
         if (vto_) cudaFree(vto_);
         vto_ = wocc_ = nullptr;
+        if (jac_) cudaFree(jac_);
+        if (vlast_) cudaFree(vlast_);
+        jac_ = vlast_ = nullptr;
+        jac_n_ = 0;
         if (Kref_) cudaFree(Kref_);
         if (Cref_) cudaFree(Cref_);
         if (Wq_) cudaFree(Wq_);
@@ -1038,6 +1076,8 @@ class ScfRun {
     double *Kref_ = nullptr, *Cref_ = nullptr, *Wq_ = nullptr, *core_ = nullptr;   // incremental Fock state
     bool late_ = false;            // past the max|e| < 1e-4 point (split: the 5-slice builds)
     double* abuf_ = nullptr;       // approximate diagonalisation scratch
+    double *jac_ = nullptr, *vlast_ = nullptr;   // Jacobi work space; last eigenvectors (and a product) of eig_from_last
+    int jac_n_ = 0;
     float *f32a_ = nullptr, *f32w_ = nullptr, *f32work_ = nullptr;   // FP32 eigensolve: matrix, values, workspace
     int f32lwork_ = 0;
     bool mixed_step_ = false;      // the last full Roothaan step was the FP32 eigensolve with FP64 refinement
