@@ -1,7 +1,6 @@
 // The C ABI (include/dfhf.h): handle set-up, shell tables, B construction and the public entry
 // points. Every entry point converts internal exceptions into status codes.
 #include <algorithm>
-#include <chrono>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -235,94 +234,83 @@ void tri_inv_lower(cudaStream_t s, double* L, int m, long long ld, double* T, co
     tri_inv_lower(s, L22, m2, ld, T, inv + (long long)m1 * 64);
 }
 
+// B of the handle's geometry. The host waits once, at the end: a factorisation that fails is reported then and its
+// B dropped. An earlier B of the handle gives its memory to the new integrals. Waits after the integrals, potrf and the
+// inverse and a buffer for each of them cost 0.5 of 13.4 ms at 4 waters (FP64) and 2.8 of 62.8 ms at 12 (split).
 void build_B(df_handle* h, double tau, bool keep, int whitening) {
     cudaStream_t s = h->stream;
     const size_t rows = (size_t)h->naux * h->pk.row;
-    cudaEvent_t ev[4];
-    for (auto& e : ev) DF_CUDA(cudaEventCreate(&e));
-    h->B.release();
+    struct Events {
+        cudaEvent_t e[5] = {};
+        ~Events() {
+            for (auto& x : e)
+                if (x) cudaEventDestroy(x);
+        }
+    } events;
+    cudaEvent_t* ev = events.e;
+    for (auto& e : events.e) DF_CUDA(cudaEventCreate(&e));
     const bool have_3c = h->a3c_ready && h->A3c.p && h->A3c.n == rows;
     h->a3c_ready = false;
+    h->built = false;
     if (!have_3c) {
-        h->A3c.release();
-        h->A3c.alloc(rows);
+        if (h->A3c.n != rows && h->B.n == rows) h->A3c = std::move(h->B);
+        else h->A3c.ensure(rows);
     }
+    if (!keep) h->B.release();
     DF_CUDA(cudaEventRecord(ev[0], s));
     if (!have_3c) compute_three_center(h, h->A3c.p, tau);
     DF_CUDA(cudaEventRecord(ev[1], s));
     // metric Cholesky (P|Q) = L L^T: cuSOLVER works column-major, so the upper factor U (V = U^T U)
     // of the column-major matrix is the row-major lower factor L = U^T (trtri of U would give L^-1).
     const int na = h->naux;
-    h->Linv.alloc((size_t)na * na);
+    h->Linv.ensure((size_t)na * na);
     DF_CUDA(cudaMemcpyAsync(h->Linv.p, h->metric.p, sizeof(double) * na * na, cudaMemcpyDeviceToDevice, s));
     int lwork = 0;
     DF_SOLVER(cusolverDnDpotrf_bufferSize(h->solver, CUBLAS_FILL_MODE_UPPER, na, h->Linv.p, na, &lwork));
-    double* work = nullptr;
-    int* info = nullptr;
-    DF_CUDA(cudaMalloc((void**)&work, sizeof(double) * std::max(lwork, 1)));
-    DF_CUDA(cudaMalloc((void**)&info, sizeof(int)));
-    int hinfo = 0;
-    try {
-        DF_CUDA(cudaStreamSynchronize(s));   // the integral kernels ahead on the stream are not potrf's time
-        const auto tp0 = std::chrono::steady_clock::now();
-        DF_SOLVER(cusolverDnDpotrf(h->solver, CUBLAS_FILL_MODE_UPPER, na, h->Linv.p, na, work, lwork, info));
-        DF_CUDA(cudaMemcpyAsync(&hinfo, info, sizeof(int), cudaMemcpyDeviceToHost, s));
-        DF_CUDA(cudaStreamSynchronize(s));
-        if (hinfo != 0) throw Error{DF_E_NUMERIC, "metric (P|Q) is not positive definite (potrf info " + std::to_string(hinfo) + ")"};
-        const auto tp1 = std::chrono::steady_clock::now();
-        h->timings_ms[17] = std::chrono::duration<double, std::milli>(tp1 - tp0).count();   // potrf
-        // the factor's inverse by blocks (FP64 products); DFHF_TRTRI=cusolver selects cuSOLVER's trtri, whose
-        // first call in a process was measured at up to 0.9 s (4384 functions) against 0.08-0.14 s here
-        const char* tri = std::getenv("DFHF_TRTRI");
-        if (!(tri && std::string(tri) == "cusolver")) {
-            // the row-major lower factor: zero its upper triangle, then invert by blocks
-            zero_upper_kernel<<<(unsigned)(((long long)na * na + 255) / 256), 256, 0, s>>>(h->Linv.p, na);
-            DF_CHECK_LAUNCH();
-            const int nblk = (na + 63) / 64;
-            DevBuf<double> T, inv;
-            T.alloc((size_t)((na / 2 + 63) / 64 * 64) * (size_t)(na / 2 + 64));
-            inv.alloc((size_t)nblk * 64 * 64);
-            tri_inv_blocks_kernel<<<dim3(4, nblk), 128, 0, s>>>(h->Linv.p, na, na, inv.p);
-            DF_CHECK_LAUNCH();
-            tri_inv_lower(s, h->Linv.p, na, na, T.p, inv.p);
-            DF_CUDA(cudaStreamSynchronize(s));
-        } else {
-            size_t dws = 0, hws = 0;
-            DF_SOLVER(cusolverDnXtrtri_bufferSize(h->solver, CUBLAS_FILL_MODE_UPPER, CUBLAS_DIAG_NON_UNIT, na, CUDA_R_64F,
-                                                  h->Linv.p, na, &dws, &hws));
-            void* dbuf = nullptr;
-            std::vector<char> hbuf(std::max<size_t>(hws, 1));
-            DF_CUDA(cudaMalloc(&dbuf, std::max<size_t>(dws, 1)));
-            cusolverStatus_t st = cusolverDnXtrtri(h->solver, CUBLAS_FILL_MODE_UPPER, CUBLAS_DIAG_NON_UNIT, na, CUDA_R_64F,
-                                                   h->Linv.p, na, dbuf, dws, hbuf.data(), hws, info);
-            DF_CUDA(cudaMemcpyAsync(&hinfo, info, sizeof(int), cudaMemcpyDeviceToHost, s));
-            DF_CUDA(cudaStreamSynchronize(s));
-            cudaFree(dbuf);
-            if (st != CUSOLVER_STATUS_SUCCESS) throw Error{DF_E_CUDA, "cusolverDnXtrtri failed"};
-        }
-        h->timings_ms[18] = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - tp1).count();
-        if (hinfo != 0) throw Error{DF_E_NUMERIC, "metric Cholesky factor is singular"};
-    } catch (...) {
-        cudaFree(work);
-        cudaFree(info);
-        throw;
+    // one work space: potrf's, then scratch and the diagonal blocks' inverses of the triangular inverse, the
+    // status words behind them
+    const int nblk = (na + 63) / 64;
+    const size_t half = (size_t)((na / 2 + 63) / 64 * 64) * (size_t)(na / 2 + 64);
+    DevBuf<double> wbuf;
+    wbuf.alloc(std::max((size_t)std::max(lwork, 1), half + (size_t)nblk * 64 * 64) + 1);
+    double* work = wbuf.p;
+    int* info = reinterpret_cast<int*>(wbuf.p + wbuf.n - 1);
+    DF_CUDA(cudaMemsetAsync(info, 0, 2 * sizeof(int), s));
+    DF_SOLVER(cusolverDnDpotrf(h->solver, CUBLAS_FILL_MODE_UPPER, na, h->Linv.p, na, work, lwork, info));
+    DF_CUDA(cudaEventRecord(ev[2], s));
+    // the factor's inverse by blocks (FP64 products); DFHF_TRTRI=cusolver selects cuSOLVER's trtri, whose
+    // first call in a process was measured at up to 0.9 s (4384 functions)
+    const char* tri = std::getenv("DFHF_TRTRI");
+    if (!(tri && std::string(tri) == "cusolver")) {
+        // the row-major lower factor: zero its upper triangle, then invert by blocks
+        zero_upper_kernel<<<(unsigned)(((long long)na * na + 255) / 256), 256, 0, s>>>(h->Linv.p, na);
+        DF_CHECK_LAUNCH();
+        tri_inv_blocks_kernel<<<dim3(4, nblk), 128, 0, s>>>(h->Linv.p, na, na, work + half);
+        DF_CHECK_LAUNCH();
+        tri_inv_lower(s, h->Linv.p, na, na, work, work + half);
+    } else {
+        size_t dws = 0, hws = 0;
+        DF_SOLVER(cusolverDnXtrtri_bufferSize(h->solver, CUBLAS_FILL_MODE_UPPER, CUBLAS_DIAG_NON_UNIT, na, CUDA_R_64F,
+                                              h->Linv.p, na, &dws, &hws));
+        std::vector<char> hbuf(std::max<size_t>(hws, 1));
+        DevBuf<char> dbuf;
+        dbuf.alloc(std::max<size_t>(dws, 1));
+        const cusolverStatus_t st = cusolverDnXtrtri(h->solver, CUBLAS_FILL_MODE_UPPER, CUBLAS_DIAG_NON_UNIT, na, CUDA_R_64F,
+                                                     h->Linv.p, na, dbuf.p, dws, hbuf.data(), hws, info + 1);
+        DF_CUDA(cudaStreamSynchronize(s));   // the buffers are released here
+        if (st != CUSOLVER_STATUS_SUCCESS) throw Error{DF_E_CUDA, "cusolverDnXtrtri failed"};
     }
-    cudaFree(work);
-    cudaFree(info);
     zero_upper_kernel<<<(unsigned)(((long long)na * na + 255) / 256), 256, 0, s>>>(h->Linv.p, na);
     DF_CHECK_LAUNCH();
-    DF_CUDA(cudaEventRecord(ev[2], s));
+    DF_CUDA(cudaEventRecord(ev[3], s));
     const char* wenv = std::getenv("DFHF_WHITEN");
     if (whitening == DF_WHITEN_FP64) {
         // FP64 product on the FP64 pipe, in place by 64-row blocks of L^-1 (a copy first if A is kept)
         if (keep) {
-            h->B.alloc(rows);
+            h->B.ensure(rows);
             DF_CUDA(cudaMemcpyAsync(h->B.p, h->A3c.p, sizeof(double) * rows, cudaMemcpyDeviceToDevice, s));
         } else {
-            h->B.p = h->A3c.p;
-            h->B.n = h->A3c.n;
-            h->A3c.p = nullptr;
-            h->A3c.n = 0;
+            h->B = std::move(h->A3c);
         }
         whiten_fp64_inplace(s, na, h->n, h->Linv.p, h->B.p, h->pk.row);
     } else if (wenv && std::string(wenv) == "ff") {
@@ -333,23 +321,33 @@ void build_B(df_handle* h, double tau, bool keep, int whitening) {
         whiten_float_float(s, na, h->pk.row, h->Linv.p, lff.p, h->A3c.p, h->B.p, h->pk.row, keep);
         DF_CUDA(cudaStreamSynchronize(s));
         lff.release();
-    } else if (keep) {
-        h->B.alloc(rows);
-        whiten_ozaki(s, na, h->n, h->pk.row, h->Linv.p, h->A3c.p, h->B.p);
     } else {
-        // in place: the unwhitened tensor's memory becomes B
-        whiten_ozaki(s, na, h->n, h->pk.row, h->Linv.p, h->A3c.p, h->A3c.p);
-        h->B.p = h->A3c.p;
-        h->B.n = h->A3c.n;
-        h->A3c.p = nullptr;
-        h->A3c.n = 0;
+        if (keep) {
+            h->B.ensure(rows);
+            whiten_ozaki(s, na, h->n, h->pk.row, h->Linv.p, h->A3c.p, h->B.p);
+        } else {
+            // in place: the unwhitened tensor's memory becomes B
+            whiten_ozaki(s, na, h->n, h->pk.row, h->Linv.p, h->A3c.p, h->A3c.p);
+            h->B = std::move(h->A3c);
+        }
     }
-    DF_CUDA(cudaEventRecord(ev[3], s));
-    DF_CUDA(cudaEventSynchronize(ev[3]));
+    DF_CUDA(cudaEventRecord(ev[4], s));
+    int hinfo[2] = {0, 0};
+    DF_CUDA(cudaMemcpyAsync(hinfo, info, sizeof hinfo, cudaMemcpyDeviceToHost, s));
+    DF_CUDA(cudaStreamSynchronize(s));
+    if (hinfo[0] != 0) {
+        h->B.release();
+        throw Error{DF_E_NUMERIC, "metric (P|Q) is not positive definite (potrf info " + std::to_string(hinfo[0]) + ")"};
+    }
+    if (hinfo[1] != 0) {
+        h->B.release();
+        throw Error{DF_E_NUMERIC, "metric Cholesky factor is singular"};
+    }
     h->timings_ms[1] = elapsed_ms(ev[0], ev[1]);
-    h->timings_ms[2] = elapsed_ms(ev[1], ev[2]);
-    h->timings_ms[3] = elapsed_ms(ev[2], ev[3]);
-    for (auto& e : ev) cudaEventDestroy(e);
+    h->timings_ms[2] = elapsed_ms(ev[1], ev[3]);
+    h->timings_ms[3] = elapsed_ms(ev[3], ev[4]);
+    h->timings_ms[17] = elapsed_ms(ev[1], ev[2]);   // potrf
+    h->timings_ms[18] = elapsed_ms(ev[2], ev[3]);   // inverse
     if (!keep) h->A3c.release();
     h->built = true;
     h->whitening = whitening;

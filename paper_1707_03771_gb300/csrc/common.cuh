@@ -107,6 +107,10 @@ struct DevBuf {
         DF_CUDA(cudaMalloc((void**)&p, count * sizeof(T)));
         n = count;
     }
+    // `count` elements: the present allocation where it is of that size, else a new one
+    void ensure(size_t count) {
+        if (n != count) alloc(count);
+    }
     void zero(cudaStream_t s) {
         if (p) DF_CUDA(cudaMemsetAsync(p, 0, n * sizeof(T), s));
     }
