@@ -2,13 +2,14 @@
 // Luk, SIAM J. Sci. Stat. Comput. 6, 69 (1985)) as one cooperative kernel.
 //
 // cuSOLVER's dsyevd takes 4.0 ms for n = 100 (a hundred-odd dependent launches); an SCF of two waters spent three
-// quarters of its time there. Here a step of the round-robin order rotates n / 2 disjoint pairs at once: every
-// CTA forms all rotations of the step itself from the current matrix, the 2 x 2 blocks (pair x pair, half of them
-// by symmetry) and the eigenvectors' elements are dealt to the threads, the new matrix goes to a second buffer,
-// and a grid barrier ends the step. A step is a few L2 latencies and the barrier, about 3 us; a sweep has n - 1
-// steps, and a matrix that is nearly diagonal (an SCF's Fock matrix in the last iteration's orbitals) needs three
-// or four. The angle is taken in FP32 (it only has to make the element small), the rotation is orthogonal to FP64
-// rounding: c = (1 + t^2)^(-1/2) by one third-order step from the FP32 value, s = t c.
+// quarters of its time there (93.6 ms, now 33.9; a solve 1.14 ms on average). Here a step of the round-robin order
+// rotates n / 2 disjoint pairs at once: every CTA forms all rotations of the step itself from the current matrix,
+// the 2 x 2 blocks (pair x pair, half of them by symmetry) and the eigenvectors' elements are dealt to the threads,
+// the new matrix goes to a second buffer, and a grid barrier ends the step. A step is a few L2 latencies and the
+// barrier, 3.4 us at n = 100; a sweep has n - 1 steps, and a matrix that is nearly diagonal (an SCF's Fock matrix in
+// the last iteration's orbitals) needs three or four. The angle is taken in FP32 (it only has to make the element
+// small), the rotation is orthogonal to FP64 rounding: c = (1 + t^2)^(-1/2) by one third-order step from the FP32
+// value, s = t c.
 #include "common.cuh"
 #include "grid_barrier.cuh"
 
@@ -215,7 +216,7 @@ void jacobi_eig(cudaStream_t s, int n, const double* A, double* w, double* out, 
     DF_CUDA(cudaMemsetAsync(info, 0, sizeof(int), s));
     JacobiArgs a{n, A, work, work + nn, work + 2 * nn, out, w, sync, info, info};
     const int m = (n + 1) / 2, tasks = m * (m + 1) + m * n;
-    const int grid = (tasks + JT - 1) / JT;   // 151 at n = 160: one CTA per SM at most
+    const int grid = (tasks + JT - 1) / JT;   // 236 at n = 200: two CTAs per SM
     void* args[] = {&a};
     DF_CUDA(cudaLaunchCooperativeKernel((const void*)jacobi_kernel, dim3(grid), dim3(JT), args, 0, s));
 }

@@ -25,7 +25,8 @@ def _system(waters, drop):
     return clusters.System(atoms=s.atoms, basis=s.basis[:len(s.basis) - drop], aux=s.aux, label=f"{s.label}-{drop}")
 
 
-@pytest.mark.parametrize("waters,drop", [(1, 0), (1, 1), (1, 2), (2, 0), (2, 3), (3, 0), (3, 2), (4, 0)])
+@pytest.mark.parametrize("waters,drop", [(1, 0), (1, 1), (1, 2), (2, 0), (2, 3), (3, 0), (3, 2), (4, 0), (4, 3), (5, 0), (5, 1),
+                                         (6, 0)])
 def test_orbitals_of_a_converged_run(lib, waters, drop):
     system = _system(waters, drop)
     with lib.Handle(system) as h:
