@@ -42,10 +42,10 @@ namespace {
 // forward, one per layer but the first backward, and one more. Parameter updates (the weight gradient of a
 // few outputs, consumed by Adam as it is formed) ride along in the phases after the one that last reads the
 // weights. Samples are read through the epoch's permutation. A phase is a few L2 latencies long, so tiles are as
-// narrow as the CTAs allow (16 rows x 2 to 16 columns, the contraction dealt to groups of threads), and a tile's
-// whole operands are requested at once.
-// Measured: 4 epochs of 17 steps, 57-256-256-256-1275, 16 samples: 36.5 -> 3.5 ms (44 us a step, of which
-// the eight barriers take 8, the weight updates with their quotients and square roots 13).
+// narrow as the CTAs allow (16 rows x 2 to 16 columns), and a tile's whole operands are requested at once.
+// Measured: 4 epochs of 17 steps, 57-256-256-256-1275, 16 samples: 37.7 -> 3.9 ms (of a step, about 50 us,
+// the eight barriers take 8 and the weight updates with their quotients and square roots 13). Every number is that
+// of the same sums and updates done one by one in ascending order, bit for bit.
 // ---------------------------------------------------------------------------------------------
 constexpr int NT = 256;             // threads of a CTA
 constexpr int STAGE_BYTES = 104 * 1024;   // shared memory of a tile's operands (two CTAs fit an SM)
@@ -73,8 +73,8 @@ struct StepArgs {
     const int* perm;                // sample of row r of step t: perm[t rows + r] (null: r)
     float scale;                    // 1 / (rows nout)
     float* part;                    // loss partials, 256 per step
-    const float2* c;                // learning rate and bias corrections per step (adam_update)
-    float b1, b2, eps;
+    const float4* c;                // bias corrections per step (adam_update)
+    float lr, b1, b2, eps;
     unsigned* count;                // barrier arrivals
     int* err;
 };
@@ -96,23 +96,24 @@ __device__ __forceinline__ void stage_row(float* dst, const float* src, int kc, 
     }
 }
 
-// one tile of 16 rows x W columns of sum_k A[r][k] B(k, n): thread (row, column, group) sums the group's part
-// (one in 16 / W) of the staged elements, the groups' sums are added through shared memory and thread
-// tid < 16 W gets element (tid / W, tid % W). A rows through `row` (offset of row r of the tile, or -1); BT:
+// one tile of 16 rows x W columns of sum_k A[r][k] B(k, n): all threads stage the operands, thread tid < 16 W sums
+// element (tid / W, tid % W), one chain of multiply-adds in ascending k whatever the tile. (Dealt to groups of threads
+// the sum is shorter by 0.4 us a phase of 256, but its rounding then depends on the tile; and where a
+// pre-activation is within rounding of zero the sign decides a sample's gradient, which Adam's first steps turn
+// into changes of the size of the learning rate.) A rows through `row` (offset of row r of the tile, or -1); BT:
 // B(k, n) = B[n ldb + k], else B[k ldb + n]. (What other CTAs wrote is visible after the barrier's acquire.)
 template <int W, bool BT, typename Row>
-__device__ float tile_sum(const float* A, Row row, const float* B, long long ldb, int n0, int nn, int K, float* stage,
-                          float* red) {
-    constexpr int G = 16 / W, KC = stage_k<W>();
+__device__ float tile_sum(const float* A, Row row, const float* B, long long ldb, int n0, int nn, int K, float* stage) {
+    constexpr int KC = stage_k<W>();
     constexpr int KP = KC + 4;      // padded row: 16-byte reads of eight rows fall on distinct banks
     const int tid = threadIdx.x;
     float* As = stage;              // [16][KP]
     float* Bs = stage + 16 * KP;    // BT: [W][KP], else [KC][W]
     float s = 0.f;
-    const int n = tid % W, r = tid / W % 16, g = tid / (16 * W);
+    const int n = tid % W, r = tid / W % 16;
     for (int k0 = 0; k0 < K; k0 += KC) {
         const int kc = min(KC, K - k0);
-        const int kg = ((kc + G - 1) / G + 3) / 4 * 4, kz = min(KC, kg * G);   // elements up to kz are read
+        const int kz = (kc + 3) / 4 * 4;   // elements up to kz are read
         __syncthreads();
         const int warp = tid >> 5, lane = tid & 31;
 #pragma unroll
@@ -138,9 +139,9 @@ __device__ float tile_sum(const float* A, Row row, const float* B, long long ldb
         }
         asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
         __syncthreads();
-        const int ke = min(kz, (g + 1) * kg);
+        if (tid >= 16 * W) continue;
 #pragma unroll 8
-        for (int k = g * kg; k < ke; k += 4) {
+        for (int k = 0; k < kz; k += 4) {
             const float4 x = *reinterpret_cast<const float4*>(As + r * KP + k);
             float4 y;
             if (BT) y = *reinterpret_cast<const float4*>(Bs + n * KP + k);
@@ -151,32 +152,39 @@ __device__ float tile_sum(const float* A, Row row, const float* B, long long ldb
             s = fmaf(x.w, y.w, s);
         }
     }
-    if (G == 1) return s;
-    red[tid] = s;
-    __syncthreads();
-    if (tid < 16 * W)
-        for (int q = 1; q < G; ++q) s += red[q * 16 * W + tid];
     return s;
 }
 
 template <bool BT, typename Row>
 __device__ float tile_sum_w(int W, const float* A, Row row, const float* B, long long ldb, int n0, int nn, int K,
-                            float* stage, float* red) {
+                            float* stage) {
     switch (W) {
-        case 16: return tile_sum<16, BT>(A, row, B, ldb, n0, nn, K, stage, red);
-        case 8: return tile_sum<8, BT>(A, row, B, ldb, n0, nn, K, stage, red);
-        case 4: return tile_sum<4, BT>(A, row, B, ldb, n0, nn, K, stage, red);
-        default: return tile_sum<2, BT>(A, row, B, ldb, n0, nn, K, stage, red);
+        case 16: return tile_sum<16, BT>(A, row, B, ldb, n0, nn, K, stage);
+        case 8: return tile_sum<8, BT>(A, row, B, ldb, n0, nn, K, stage);
+        case 4: return tile_sum<4, BT>(A, row, B, ldb, n0, nn, K, stage);
+        default: return tile_sum<2, BT>(A, row, B, ldb, n0, nn, K, stage);
     }
 }
 
-// Adam (Kingma & Ba 2015) with bias correction: p -= lr (m / c1) / (sqrt(v / c2) + eps), c = (lr / c1, 1 / sqrt(c2))
-__device__ __forceinline__ void adam_update(float& p, float g, float& m, float& v, float b1, float b2, float eps, float2 c) {
-    const float mi = b1 * m + (1.f - b1) * g;
-    const float vi = b2 * v + (1.f - b2) * g * g;
+// a / b from y = 1 / b correctly rounded: q = a y is within a unit in the last place, and q + (a - q b) y rounds to the
+// quotient (Markstein, IBM J. Res. Dev. 34, 111 (1990)) unless b's mantissa is all ones (y = 0 is passed then) or the
+// remainder underflows, where |a| is too small to move a parameter
+__device__ __forceinline__ float quotient(float a, float b, float y) {
+    if (y == 0.f) return a / b;
+    const float q = a * y;
+    return fmaf(fmaf(-q, b, a), y, q);
+}
+
+// Adam (Kingma & Ba 2015) with bias correction: p -= lr (m / c1) / (sqrt(v / c2) + eps), c = (c1, 1 / c1, c2, 1 / c2)
+__device__ __forceinline__ void adam_update(float& p, float g, float& m, float& v, float lr, float b1, float b2, float eps,
+                                            float4 c) {
+    // the roundings are written out: they do not depend on how this code is compiled into the step kernel
+    const float mi = __fmaf_rn(1.f - b1, g, __fmul_rn(b1, m));
+    const float vi = __fmaf_rn(__fmul_rn(1.f - b2, g), g, __fmul_rn(b2, v));
     m = mi;
     v = vi;
-    p -= c.x * mi / (sqrtf(vi) * c.y + eps);
+    p = __fsub_rn(p, __fdiv_rn(__fmul_rn(lr, quotient(mi, c.x, c.y)),
+                               __fadd_rn(__fsqrt_rn(quotient(vi, c.z, c.w)), eps)));
 }
 
 __global__ void __launch_bounds__(NT, 2) mlp_steps_kernel(const StepArgs s) {
@@ -201,7 +209,7 @@ __global__ void __launch_bounds__(NT, 2) mlp_steps_kernel(const StepArgs s) {
 
     for (int step = 0; step < s.nsteps; ++step) {
         const int* perm = s.perm ? s.perm + (long long)step * s.rows : nullptr;
-        const float2 c = s.c ? s.c[step] : make_float2(1.f, 1.f);
+        const float4 c = s.c ? s.c[step] : make_float4(1.f, 1.f, 1.f, 1.f);
         __syncthreads();   // the last step's samples are no longer read
         if (tid < s.rows) sperm[tid] = perm ? __ldg(perm + tid) : tid;
         __syncthreads();
@@ -222,7 +230,7 @@ __global__ void __launch_bounds__(NT, 2) mlp_steps_kernel(const StepArgs s) {
                 const bool mine = tid < 16 * W && r < s.rows && n < y.no;
                 const float bias = mine ? __ldcg(s.P + y.b + n) : 0.f;
                 const float goal = mine && l == s.L - 1 && s.Y ? __ldg(s.Y + (long long)sample(r) * y.no + n) : 0.f;
-                const float sum = tile_sum_w<true>(W, in, row, s.P + y.w, y.ni, n0, y.no, y.ni, stage, red);
+                const float sum = tile_sum_w<true>(W, in, row, s.P + y.w, y.ni, n0, y.no, y.ni, stage);
                 if (mine) {
                     const long long at = (long long)r * y.no + n;
                     const float z = sum + bias;
@@ -285,7 +293,7 @@ __global__ void __launch_bounds__(NT, 2) mlp_steps_kernel(const StepArgs s) {
                         if (s.G) {
                             s.G[at] = g[q];
                         } else {
-                            adam_update(p[q], g[q], m[q], v[q], s.b1, s.b2, s.eps, c);
+                            adam_update(p[q], g[q], m[q], v[q], s.lr, s.b1, s.b2, s.eps, c);
                             s.P[at] = p[q];
                             s.Mom[at] = m[q];
                             s.Vel[at] = v[q];
@@ -297,7 +305,7 @@ __global__ void __launch_bounds__(NT, 2) mlp_steps_kernel(const StepArgs s) {
                     s.G[at] = gb;
                 } else {
                     float pb = __ldcg(s.P + at), mb = __ldcg(s.Mom + at), vb = __ldcg(s.Vel + at);
-                    adam_update(pb, gb, mb, vb, s.b1, s.b2, s.eps, c);
+                    adam_update(pb, gb, mb, vb, s.lr, s.b1, s.b2, s.eps, c);
                     s.P[at] = pb;
                     s.Mom[at] = mb;
                     s.Vel[at] = vb;
@@ -349,7 +357,7 @@ __global__ void __launch_bounds__(NT, 2) mlp_steps_kernel(const StepArgs s) {
                     const bool mine = tid < 16 * W && r < s.rows && n < y.ni;
                     const long long at = (long long)r * y.ni + n;
                     const float z = mine ? __ldcg(x.Z + at) : 0.f;
-                    const float sum = tile_sum_w<false>(W, y.dZ, row, s.P + y.w, y.ni, n0, y.ni, y.no, stage, red);
+                    const float sum = tile_sum_w<false>(W, y.dZ, row, s.P + y.w, y.ni, n0, y.ni, y.no, stage);
                     if (mine) x.dZ[at] = z <= 0.f ? 0.f : sum;
                 } else if (t < below + above) {
                     if (l == s.L - 1) loss_block(t - below);
@@ -427,6 +435,12 @@ struct Work {
         DF_CUDA(cudaStreamSynchronize(m->stream));   // the host array is released on return
     }
 };
+
+// 1 / b for quotient()
+inline float recip(float b) {
+    int e = 0;
+    return std::frexp(b, &e) == 1.f - 0x1p-24f ? 0.f : 1.f / b;
+}
 
 // runs a.nsteps steps (at most Work::MAX_STEPS) on two CTAs per SM; synchronises
 void run_steps(df_mlp* m, Work& w, StepArgs a) {
@@ -794,11 +808,11 @@ int df_mlp_train(df_mlp* m, const float* X, const float* Y, int ns, int epochs, 
         Work w;
         w.alloc(m, batch, chunk);
         DevBuf<int> perm;
-        DevBuf<float2> corr;
+        DevBuf<float4> corr;
         perm.alloc((size_t)chunk * batch);
         corr.alloc(chunk);
         std::vector<int> order(ns), hperm((size_t)chunk * batch);
-        std::vector<float2> hcorr(chunk);
+        std::vector<float4> hcorr(chunk);
         std::vector<float> part((size_t)256 * chunk);
         std::vector<double> ep_loss(epochs, 0.0);
         std::mt19937_64 gen(seed);
@@ -812,10 +826,10 @@ int df_mlp_train(df_mlp* m, const float* X, const float* Y, int ns, int epochs, 
                 ++m->adam_t;
                 const float b1 = 0.9f, b2 = 0.999f;
                 const float c1 = 1.f - std::pow(b1, (float)m->adam_t), c2 = 1.f - std::pow(b2, (float)m->adam_t);
-                hcorr[t] = make_float2((float)((double)lr / c1), (float)(1.0 / std::sqrt((double)c2)));
+                hcorr[t] = make_float4(c1, recip(c1), c2, recip(c2));
             }
             DF_CUDA(cudaMemcpyAsync(perm.p, hperm.data(), sizeof(int) * nt * batch, cudaMemcpyHostToDevice, m->stream));
-            DF_CUDA(cudaMemcpyAsync(corr.p, hcorr.data(), sizeof(float2) * nt, cudaMemcpyHostToDevice, m->stream));
+            DF_CUDA(cudaMemcpyAsync(corr.p, hcorr.data(), sizeof(float4) * nt, cudaMemcpyHostToDevice, m->stream));
             StepArgs a{};
             a.nsteps = nt;
             a.Mom = m->Mom.p;
@@ -824,6 +838,7 @@ int df_mlp_train(df_mlp* m, const float* X, const float* Y, int ns, int epochs, 
             a.Y = dY.p;
             a.perm = perm.p;
             a.c = corr.p;
+            a.lr = lr;
             run_steps(m, w, a);
             DF_CUDA(cudaMemcpyAsync(part.data(), w.part.p, sizeof(float) * 256 * nt, cudaMemcpyDeviceToHost, m->stream));
             DF_CUDA(cudaStreamSynchronize(m->stream));
