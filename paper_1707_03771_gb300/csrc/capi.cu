@@ -235,8 +235,10 @@ void tri_inv_lower(cudaStream_t s, double* L, int m, long long ld, double* T, co
 }
 
 // B of the handle's geometry. The host waits once, at the end: a factorisation that fails is reported then and its
-// B dropped. An earlier B of the handle gives its memory to the new integrals. Waits after the integrals, potrf and the
-// inverse and a buffer for each of them cost 0.5 of 13.4 ms at 4 waters (FP64) and 2.8 of 62.8 ms at 12 (split).
+// B dropped. An earlier B of the handle gives its memory to the new integrals, once nothing on the device reads it any
+// more: df_coulomb_noalloc returns with its reads queued, on a stream that need not be the handle's any longer. Waits
+// after the integrals, potrf and the inverse and a buffer for each of them cost 0.5 of 13.4 ms at 4 waters (FP64) and
+// 2.8 of 62.8 ms at 12 (split).
 void build_B(df_handle* h, double tau, bool keep, int whitening) {
     cudaStream_t s = h->stream;
     const size_t rows = (size_t)h->naux * h->pk.row;
@@ -252,6 +254,7 @@ void build_B(df_handle* h, double tau, bool keep, int whitening) {
     const bool have_3c = h->a3c_ready && h->A3c.p && h->A3c.n == rows;
     h->a3c_ready = false;
     h->built = false;
+    if (h->B.p) DF_CUDA(cudaDeviceSynchronize());
     if (!have_3c) {
         if (h->A3c.n != rows && h->B.n == rows) h->A3c = std::move(h->B);
         else h->A3c.ensure(rows);
