@@ -2,16 +2,26 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cstdlib>
+
 #include "../../include/dfhf.h"
 
 namespace dfhf {
 
 constexpr long long GRID_WAIT_CYCLES = 4000000000LL;   // about 2 s
 
-// count: arrivals, zero at the start of the launch; target: this CTA's running target, zero at the start.
-// False on every thread if the wait expires here or err is set elsewhere. What a CTA wrote before the barrier is
-// visible to every CTA after it.
-__device__ inline bool grid_barrier(unsigned* count, int* err, unsigned& target) {
+// Budget of a barrier's wait: GRID_WAIT_CYCLES, or DFHF_GRID_WAIT_CYCLES (a test knob that makes the waits run out,
+// to exercise the DF_E_TIMEOUT path)
+inline long long grid_wait_cycles() {
+    const char* v = std::getenv("DFHF_GRID_WAIT_CYCLES");
+    const long long c = v ? std::atoll(v) : 0;
+    return (c > 0 && c < GRID_WAIT_CYCLES) ? c : GRID_WAIT_CYCLES;
+}
+
+// count: arrivals, zero at the start of the launch; target: this CTA's running target, zero at the start; wait: the
+// budget in cycles. False on every thread if the wait expires here or err is set elsewhere. What a CTA wrote before
+// the barrier is visible to every CTA after it.
+__device__ inline bool grid_barrier(unsigned* count, int* err, unsigned& target, long long wait) {
     __shared__ int ok;
     __syncthreads();
     target += gridDim.x;
@@ -24,7 +34,7 @@ __device__ inline bool grid_barrier(unsigned* count, int* err, unsigned& target)
             unsigned seen;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(seen) : "l"(count) : "memory");
             if ((int)(seen - target) >= 0) break;
-            if (clock64() - t0 > GRID_WAIT_CYCLES || *(volatile int*)err) {
+            if (clock64() - t0 > wait || *(volatile int*)err) {
                 atomicExch(err, DF_E_TIMEOUT);
                 good = 0;
                 break;

@@ -77,6 +77,7 @@ struct StepArgs {
     float lr, b1, b2, eps;
     unsigned* count;                // barrier arrivals
     int* err;
+    long long wait;                 // budget of a barrier's wait
 };
 
 // kz floats of a row into shared memory (those from kc on, or all of a missing row, as zeros), by one warp: 16
@@ -243,7 +244,7 @@ __global__ void __launch_bounds__(NT, 2) mlp_steps_kernel(const StepArgs s) {
                 }
             }
             if (!s.Y && l == s.L - 1) continue;
-            if (!grid_barrier(s.count, s.err, target)) return;
+            if (!grid_barrier(s.count, s.err, target, s.wait)) return;
         }
         if (!s.Y) continue;
 
@@ -366,7 +367,7 @@ __global__ void __launch_bounds__(NT, 2) mlp_steps_kernel(const StepArgs s) {
                     update(0, t - below - above);
                 }
             }
-            if (!grid_barrier(s.count, s.err, target)) return;
+            if (!grid_barrier(s.count, s.err, target, s.wait)) return;
         }
     }
 }
@@ -455,6 +456,7 @@ void run_steps(df_mlp* m, Work& w, StepArgs a) {
     a.eps = 1e-8f;
     a.count = w.sync.p;
     a.err = reinterpret_cast<int*>(w.sync.p + 1);
+    a.wait = grid_wait_cycles();
     DF_CUDA(cudaMemsetAsync(w.sync.p, 0, 2 * sizeof(unsigned), m->stream));
     int dev = 0, sms = 0;
     DF_CUDA(cudaGetDevice(&dev));

@@ -29,10 +29,14 @@ struct JacobiArgs {
     double *M0, *M1, *V;            // work: n x n each
     double* out;                    // row j: eigenvector of w[j]
     double* w;                      // ascending
-    unsigned* count;
+    unsigned* count;                // barrier arrivals
+    int* top;                       // high word of the largest magnitude in A, zero at the start
     int* err;
     int* info;                      // 0, or 1 if MAX_SWEEPS did not suffice
+    long long wait;                 // budget of a barrier's wait
 };
+
+__device__ __forceinline__ int high_word(double v) { return __double2hiint(v) & 0x7fffffff; }
 
 __global__ void __launch_bounds__(JT) jacobi_kernel(const JacobiArgs a) {
     __shared__ double sc[MAXP], ss[MAXP];
@@ -42,12 +46,23 @@ __global__ void __launch_bounds__(JT) jacobi_kernel(const JacobiArgs a) {
     const int gt = blockIdx.x * JT + tid, gn = gridDim.x * JT;
     unsigned target = 0;
 
+    int top = 0;
     for (int e = gt; e < n * n; e += gn) {
         const int i = e / n, j = e % n;
-        a.M0[e] = a.A[i >= j ? e : j * n + i];
+        const double v = a.A[i >= j ? e : j * n + i];
+        a.M0[e] = v;
         a.V[e] = i == j ? 1.0 : 0.0;
+        top = max(top, high_word(v));
     }
-    if (!grid_barrier(a.count, a.err, target)) return;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    if ((tid & 31) == 0) atomicMax(a.top, top);
+    if (!grid_barrier(a.count, a.err, target, a.wait)) return;
+    // a matrix whose magnitude is far from 1 (the change of a density between two iterations may be) has its angles'
+    // FP32 operands scaled to the range of floats; others are taken as they are
+    top = __ldcg(a.top);
+    const bool far = top < 0x7ff00000 && abs((top >> 20) - 1023) > 60;
+    const double scale = __hiloint2double(max(1, 2046 - (top >> 20)) << 20, 0);
 
     // this thread's task in every step: one new row (the pair's first or second) of a block (I, J), I >= J, of
     // pair rows and pair columns (and its mirror image), or element tj of the eigenvectors of pair ti. The launch
@@ -75,7 +90,7 @@ __global__ void __launch_bounds__(JT) jacobi_kernel(const JacobiArgs a) {
         q = max(x, y);
     };
     double *cur = a.M0, *nxt = a.M1;
-    bool done = n == 1;
+    bool done = n == 1 || top == 0;
     for (int sweep = 0; sweep < MAX_SWEEPS && !done; ++sweep) {
         int off = 0, big = 0;                        // largest magnitudes of the sweep, as high words of doubles
         for (int t = 0; t < N1; ++t) {
@@ -100,11 +115,16 @@ __global__ void __launch_bounds__(JT) jacobi_kernel(const JacobiArgs a) {
                 double c = 1.0, s = 0.0;
                 if (q < n) {
                     const double app = __ldcg(cur + p * n + p), aqq = __ldcg(cur + q * n + q), apq = __ldcg(cur + p * n + q);
-                    off = max(off, __double2hiint(apq) & 0x7fffffff);
-                    big = max(big, max(__double2hiint(app) & 0x7fffffff, __double2hiint(aqq) & 0x7fffffff));
-                    const float f = (float)apq;
+                    off = max(off, high_word(apq));
+                    big = max(big, max(high_word(app), high_word(aqq)));
+                    double gap = aqq - app, el = apq;
+                    if (far) {
+                        gap *= scale;
+                        el *= scale;
+                    }
+                    const float f = (float)el;
                     if (f != 0.f) {
-                        const float th = (float)(aqq - app) / (2.f * f);
+                        const float th = (float)gap / (2.f * f);
                         const double tt = (double)copysignf(1.f / (fabsf(th) + sqrtf(fmaf(th, th, 1.f))), th);
                         const double x = fma(tt, tt, 1.0);
                         const double y = (double)rsqrtf((float)x);
@@ -149,7 +169,7 @@ __global__ void __launch_bounds__(JT) jacobi_kernel(const JacobiArgs a) {
                 a.V[p1 * n + tj] = fma(c1, x00, -s1 * x10);
                 a.V[q1 * n + tj] = fma(s1, x00, c1 * x10);
             }
-            if (!grid_barrier(a.count, a.err, target)) return;
+            if (!grid_barrier(a.count, a.err, target, a.wait)) return;
             double* x = cur;
             cur = nxt;
             nxt = x;
@@ -174,17 +194,17 @@ __global__ void __launch_bounds__(JT) jacobi_kernel(const JacobiArgs a) {
         // near the end (the convergence is quadratic) the elements themselves are looked at, which spares the sweep
         // that would only find them small
         const double diag = __hiloint2double(big, 0);
-        if (__hiloint2double(off, -1) > 1e-4 * diag) continue;
+        if (off && __hiloint2double(off, -1) > 1e-4 * diag) continue;
         int left = 0;
         for (int e = tid; e < n * n; e += JT)
-            if (e / n != e % n) left = max(left, __double2hiint(__ldcg(cur + e)) & 0x7fffffff);
+            if (e / n != e % n) left = max(left, high_word(__ldcg(cur + e)));
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) left = max(left, __shfl_xor_sync(0xffffffffu, left, o));
         if ((tid & 31) == 0) red_off[tid >> 5] = left;
         __syncthreads();
         for (int k = 0; k < JT / 32; ++k) left = max(left, red_off[k]);
         __syncthreads();
-        done = __hiloint2double(left, -1) <= OFF_TOL * diag;
+        done = !left || __hiloint2double(left, -1) <= OFF_TOL * diag;
     }
     // ascending order
     for (int i = tid; i < n; i += JT) {
@@ -211,10 +231,11 @@ size_t jacobi_work_doubles(int n) { return 3 * (size_t)n * n + 1; }
 // barrier that expires leaves DF_E_TIMEOUT there.
 void jacobi_eig(cudaStream_t s, int n, const double* A, double* w, double* out, double* work, int* info) {
     const size_t nn = (size_t)n * n;
-    unsigned* sync = reinterpret_cast<unsigned*>(work + 3 * nn);
-    DF_CUDA(cudaMemsetAsync(sync, 0, sizeof(unsigned), s));
+    unsigned* sync = reinterpret_cast<unsigned*>(work + 3 * nn);   // arrivals | largest magnitude
+    DF_CUDA(cudaMemsetAsync(sync, 0, 2 * sizeof(unsigned), s));
     DF_CUDA(cudaMemsetAsync(info, 0, sizeof(int), s));
-    JacobiArgs a{n, A, work, work + nn, work + 2 * nn, out, w, sync, info, info};
+    JacobiArgs a{n,    A,    work, work + nn, work + 2 * nn, out, w, sync, reinterpret_cast<int*>(sync + 1),
+                 info, info, grid_wait_cycles()};
     const int m = (n + 1) / 2, tasks = m * (m + 1) + m * n;
     const int grid = (tasks + JT - 1) / JT;   // 236 at n = 200: two CTAs per SM
     void* args[] = {&a};

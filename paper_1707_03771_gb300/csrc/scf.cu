@@ -473,7 +473,7 @@ class ScfRun {
         int hinfo = 0;
         DF_CUDA(cudaMemcpyAsync(&hinfo, info_, sizeof(int), cudaMemcpyDeviceToHost, s_));
         DF_CUDA(cudaStreamSynchronize(s_));
-        if (hinfo != 0) throw Error{DF_E_NUMERIC, "dsyevd of S failed, info " + std::to_string(hinfo)};
+        check_eig(hinfo, own_eig(n_), " of S");
         int first = 0;
         while (first < n_ && sv[first] <= 1e-7) ++first;
         nX_ = n_ - first;
@@ -642,8 +642,7 @@ class ScfRun {
         DF_CUDA(cudaEventSynchronize(ev_done_));
         const double this_jk = elapsed_ms(ej0_, ej1_);
         jk_ms_ += this_jk;
-        if (pin_ctl_[2 * DIIS_MAX + 1] != 0)
-            throw Error{DF_E_NUMERIC, "dsyevd failed, info " + std::to_string(pin_ctl_[2 * DIIS_MAX + 1])};
+        check_eig(pin_ctl_[2 * DIIS_MAX + 1], own_eig(nX_) || own_eig(2 * nocc_), "");
         if (pin_ctl_[2 * DIIS_MAX + 2] != 0)
             throw Error{DF_E_TIMEOUT, "tensor-core exchange kernel timed out waiting on a barrier"};
         if (pin_ctl_[2 * DIIS_MAX] != 0 && !order_.empty()) {   // last DIIS system was singular
@@ -821,6 +820,14 @@ class ScfRun {
     // SAD guess that starts them) keep cuSOLVER's at every size: their early 3-slice exchange depends on the last
     // bits of the orbitals, so another solver's rotations within the occupied space would show in their results.
     bool own_eig(int m) const { return o_.precision == DF_PREC_FP64 && !frac_ && m <= JACOBI_MAX; }
+
+    // throws for an eigensolve that failed; own: jacobi.cu's solver may have been the one
+    static void check_eig(int info, bool own, const char* of) {
+        if (info == 0) return;
+        if (own && info == DF_E_TIMEOUT)
+            throw Error{DF_E_TIMEOUT, "Jacobi eigensolver timed out waiting on its grid barrier"};
+        throw Error{DF_E_NUMERIC, std::string(own ? "Jacobi eigensolver" : "syevd") + of + " failed, info " + std::to_string(info)};
+    }
 
     void eig(double* A, int m, double* w) {
         if (own_eig(m)) {
@@ -1004,6 +1011,10 @@ class ScfRun {
         if (last_approx_) {
             DF_CUDA(cudaMemcpyAsync(Fp_, Fo_, sizeof(double) * nX_ * nX_, cudaMemcpyDeviceToDevice, s_));
             eig(Fp_, nX_, h_->eps.p);
+            int hinfo = 0;
+            DF_CUDA(cudaMemcpyAsync(&hinfo, info_, sizeof(int), cudaMemcpyDeviceToHost, s_));
+            DF_CUDA(cudaStreamSynchronize(s_));
+            check_eig(hinfo, own_eig(nX_), "");
         }
         if (vt_ == Fp_) mm(s_, false, true, n_, nX_, nX_, 1.0, h_->X.p, nX_, Fp_, nX_, 0.0, h_->C.p, nX_);
         done_ = true;
