@@ -769,11 +769,9 @@ void y_tc_launch(cudaStream_t s, const CUtensorMap& ma, const bf16* Cs, const Tc
     launch_tc<S, N, MODE>(s, ma, mb, mb2, a, row_tiles * ((a.cols + N - 1) / N));
 }
 
-// N: tile width; a tile is no wider than the columns (64 wide over 48 or fewer runs the 48-wide kernel, of which
-// two CTAs fit an SM)
+// N: tile width
 template <int MODE>
 void y_tc_dispatch(cudaStream_t s, int S, int N, const CUtensorMap& ma, const bf16* Cs, const TcArgs& a, long long row_tiles) {
-    if (N == 64 && a.cols <= 48) N = 48;
     if (S == 3 && N == 80) y_tc_launch<3, 80, MODE>(s, ma, Cs, a, row_tiles);
     else if (S == 5 && N == 80) y_tc_launch<5, 80, MODE>(s, ma, Cs, a, row_tiles);
     else if (S == 3 && N == 64) y_tc_launch<3, 64, MODE>(s, ma, Cs, a, row_tiles);
