@@ -11,6 +11,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <new>
 #include <random>
 #include <vector>
 
@@ -413,14 +414,19 @@ struct Work {
     DevBuf<unsigned> sync;          // barrier arrivals | error word
     float* out = nullptr;           // the last layer's outputs (rows x nout)
     int rows = 0;
-    static constexpr int MAX_STEPS = 4096;   // per launch
+    static constexpr int MAX_STEPS = 4096;                 // per launch,
+    static constexpr long long MAX_SAMPLES = 1 << 20;      // and rows of all of its steps (4 MB of indices)
+    // steps of n rows per launch
+    static int launch_steps(long long steps, int n) {
+        return (int)std::min(std::min<long long>(steps, MAX_STEPS), std::max(1LL, MAX_SAMPLES / n));
+    }
     void alloc(df_mlp* m, int n, int steps) {
         rows = n;
         const int L = (int)m->dims.size() - 1;
         size_t per = 0;
         for (int l = 0; l < L; ++l) per += m->dims[l + 1];
         buf.alloc(3 * per * n);
-        part.alloc((size_t)256 * std::min(steps, MAX_STEPS));
+        part.alloc((size_t)256 * steps);
         part.zero(m->stream);
         sync.alloc(2);
         std::vector<Layer> host(L);
@@ -790,6 +796,8 @@ int df_mlp_gradients(df_mlp* m, const float* X, const float* Y, int ns, float* g
         if (loss) *loss = step_loss(part.data());
     } catch (const Error& e) {
         return e.code;
+    } catch (const std::bad_alloc&) {
+        return DF_E_NOMEM;
     }
     return DF_OK;
 }
@@ -806,7 +814,7 @@ int df_mlp_train(df_mlp* m, const float* X, const float* Y, int ns, int epochs, 
         dY.alloc((size_t)ns * m->nout);
         DF_CUDA(cudaMemcpyAsync(dX.p, X, sizeof(float) * ns * m->nin, cudaMemcpyHostToDevice, m->stream));
         DF_CUDA(cudaMemcpyAsync(dY.p, Y, sizeof(float) * ns * m->nout, cudaMemcpyHostToDevice, m->stream));
-        const int chunk = (int)std::min<long long>(steps, Work::MAX_STEPS);
+        const int chunk = Work::launch_steps(steps, batch);
         Work w;
         w.alloc(m, batch, chunk);
         DevBuf<int> perm;
@@ -825,9 +833,8 @@ int df_mlp_train(df_mlp* m, const float* X, const float* Y, int ns, int epochs, 
                 const int b = (int)((t0 + t) % per_epoch);
                 if (b == 0) std::shuffle(order.begin(), order.end(), gen);   // a new epoch
                 for (int r = 0; r < batch; ++r) hperm[(size_t)t * batch + r] = order[b * batch + r];
-                ++m->adam_t;
-                const float b1 = 0.9f, b2 = 0.999f;
-                const float c1 = 1.f - std::pow(b1, (float)m->adam_t), c2 = 1.f - std::pow(b2, (float)m->adam_t);
+                const float b1 = 0.9f, b2 = 0.999f, at = (float)(m->adam_t + t + 1);
+                const float c1 = 1.f - std::pow(b1, at), c2 = 1.f - std::pow(b2, at);
                 hcorr[t] = make_float4(c1, recip(c1), c2, recip(c2));
             }
             DF_CUDA(cudaMemcpyAsync(perm.p, hperm.data(), sizeof(int) * nt * batch, cudaMemcpyHostToDevice, m->stream));
@@ -842,6 +849,7 @@ int df_mlp_train(df_mlp* m, const float* X, const float* Y, int ns, int epochs, 
             a.c = corr.p;
             a.lr = lr;
             run_steps(m, w, a);
+            m->adam_t += nt;
             DF_CUDA(cudaMemcpyAsync(part.data(), w.part.p, sizeof(float) * 256 * nt, cudaMemcpyDeviceToHost, m->stream));
             DF_CUDA(cudaStreamSynchronize(m->stream));
             for (int t = 0; t < nt; ++t) ep_loss[(t0 + t) / per_epoch] += step_loss(part.data() + (size_t)256 * t);
@@ -850,6 +858,8 @@ int df_mlp_train(df_mlp* m, const float* X, const float* Y, int ns, int epochs, 
             for (int ep = 0; ep < epochs; ++ep) loss_history[ep] = (float)(ep_loss[ep] / per_epoch);
     } catch (const Error& e) {
         return e.code;
+    } catch (const std::bad_alloc&) {
+        return DF_E_NOMEM;
     }
     return DF_OK;
 }
@@ -899,6 +909,8 @@ int df_mlp_predict(df_mlp* m, const float* X, int ns, int bf16, float* Y) {
         out.release();
     } catch (const Error& e) {
         return e.code;
+    } catch (const std::bad_alloc&) {
+        return DF_E_NOMEM;
     }
     return DF_OK;
 }
