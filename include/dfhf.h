@@ -235,7 +235,7 @@ int scf_run_rohf(df_handle* h, const df_options* opts, int nalpha, int nbeta, do
  * in FP64 on the GPU from the handle's B. C: host, n x nmo row-major, column k = canonical orbital k in
  * ascending energy (the first nocc occupied; e.g. df_get_matrix 10 after scf_run, nmo = n - dropped); eps:
  * host, nmo orbital energies. Requires B (DF_E_STATE), 1 <= nocc < nmo <= n (DF_E_ARG). Device memory:
- * about 8 naux (n + nvir) nocc bytes besides B. */
+ * about 8 nocc (naux nvir + max(naux n, nvir^2)) bytes besides B. */
 int df_mp2(df_handle* h, const double* C, const double* eps, int nmo, int nocc, double* e2);
 
 /* ---- density-fitting object operations (paper, section "Density fitting utilities", eqs. 1-3) ----------

@@ -9,6 +9,7 @@
 //     summed per pair and 32 x 32 tile of (a, b) in one block (fixed order), these added on the host in a
 //     fixed order.
 #include <cmath>
+#include <new>
 #include <vector>
 
 #include "common.cuh"
@@ -87,6 +88,7 @@ double mp2_energy(df_handle* h, const double* C_host, const double* eps_host, in
     // T[i][a][P] = sum_mu Y[mu][P nocc + i] C_vir[mu][a]: rows (P, i), every P in one product
     T.alloc((size_t)KL * nvir);
     dgemm_rows(s, naux, nocc, nvir, n, 1.0, Y.p, nocc, 1, KL, Cvir.p, nvir, 1, 0.0, T.p, 1, (long long)nvir * naux, naux);
+    Y.release();   // V takes its room: the peak is T and the larger of Y and V
     // rows of pair integrals: V = T_i T_{0..i}^T (nvir x (i + 1) nvir) and the pair energies of row i
     const int nt = (nvir + MT - 1) / MT, ntp = nt * (nt + 1) / 2;
     V.alloc((size_t)nvir * nocc * nvir);
@@ -123,6 +125,9 @@ extern "C" int df_mp2(df_handle* h, const double* C, const double* eps, int nmo,
     } catch (const Error& e) {
         h->last_error = e.msg;
         return e.code;
+    } catch (const std::bad_alloc&) {
+        h->last_error = "df_mp2: host memory exhausted";
+        return DF_E_NOMEM;
     }
     return DF_OK;
 }
