@@ -838,6 +838,7 @@ class ScfRun {
                 DF_CUDA(cudaMalloc((void**)&jac_, sizeof(double) * jacobi_work_doubles(jac_n_)));
             }
             jacobi_eig(s_, m, A, w, A, jac_, info_);
+            orthonormalise(A, m);
             return;
         }
         int lw = 0;
@@ -845,6 +846,18 @@ class ScfRun {
         grow_work(lw);
         DF_SOLVER(cusolverDnDsyevd(h_->solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_UPPER, m, A, m, w, work_,
                                    lwork_, info_));
+    }
+
+    // rows of V (m x m) orthonormal to rounding: a Newton-Schulz step V <- 1.5 V - 0.5 (V V^T) V, which squares the
+    // error. A Jacobi solve's rotations leave some 1e-14, and vectors that are carried from iteration to iteration add
+    // theirs up: 1.6e-12 after 400 iterations of an SCF that does not converge (n = 200), against 3e-14 from fresh
+    // solves. Scratch: the Jacobi work space, free after a solve.
+    void orthonormalise(double* V, int m) {
+        double *G = jac_, *W = jac_ + (long long)m * m;
+        mm(s_, false, true, m, m, m, 1.0, V, m, V, m, 0.0, G, m);
+        DF_CUDA(cudaMemcpyAsync(W, V, sizeof(double) * m * m, cudaMemcpyDeviceToDevice, s_));
+        mm(s_, false, false, m, m, m, -0.5, G, m, V, m, 1.5, W, m);
+        DF_CUDA(cudaMemcpyAsync(V, W, sizeof(double) * m * m, cudaMemcpyDeviceToDevice, s_));
     }
 
     // eigenvectors of the Fock matrix in Fp_ (in place) in the basis of the last iteration's (vlast_), where it is
@@ -860,6 +873,7 @@ class ScfRun {
             mm(s_, false, true, nX_, nX_, nX_, 1.0, T, nX_, vlast_, nX_, 0.0, Fp_, nX_);
             jacobi_eig(s_, nX_, Fp_, h_->eps.p, T, jac_, info_);
             mm(s_, false, false, nX_, nX_, nX_, 1.0, T, nX_, vlast_, nX_, 0.0, Fp_, nX_);
+            orthonormalise(Fp_, nX_);
         }
         DF_CUDA(cudaMemcpyAsync(vlast_, Fp_, sizeof(double) * no, cudaMemcpyDeviceToDevice, s_));
     }
