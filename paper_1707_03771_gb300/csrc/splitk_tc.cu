@@ -52,6 +52,17 @@ template <int S, int N>
 constexpr int ring_slots() {
     return (S >= 7 && N <= 32) || (S == 5 && N == 48) || (S == 3 && N == 64) ? 3 : 4;
 }
+template <int S, int N>
+constexpr int tc_smem_bytes() {
+    return ring_slots<S, N>() * TM * KS * 2 + 2 * S * N * KS * 2 + 1024 + 256;
+}
+// two CTAs share an SM where the accumulators take at most half of its tensor memory and the rings fit twice into
+// 228 KB; the kernel's registers are bounded for two there, and only there (3 slices, 80 wide: 372 bytes of spills
+// for a second CTA that has no room; Y at n = 800, naux = 2192, 80 occupied 1.86 -> 1.81 ms without)
+template <int S, int N>
+constexpr int ctas_per_sm() {
+    return S * N <= 256 && 2 * (tc_smem_bytes<S, N>() + 1024) <= 228 * 1024 ? 2 : 1;
+}
 constexpr long long WAIT_CYCLES = 4000000000LL;   // ~2 s at 2 GHz
 
 // ------------------------------------------------------------------------------------------------
@@ -296,8 +307,7 @@ __device__ __forceinline__ Tile decode_tile(const TcArgs& args, int b) {
     return t;
 }
 
-// Two CTAs share an SM where the accumulators take at most half of its tensor memory (S N <= 256 columns): one
-// drains while the other's products run. What bounds it (measured on a stream of MMAs alone): an MMA of width W
+// Where two CTAs share an SM, one drains while the other's products run. What bounds it (measured on a stream of MMAs alone): an MMA of width W
 // takes max(W / 2, (4096 + 32 W) / 128) clocks, arithmetic or the read of its shared-memory operands at 128 bytes
 // a clock, and the TMA writes of the streamed slices (16 KB of A and 128 N bytes of B per slice and K-step) share
 // that memory; so wider tiles do better, up to the 48 columns at which two CTAs still fit (5 slices: 94 % of the
@@ -309,7 +319,7 @@ __device__ __forceinline__ Tile decode_tile(const TcArgs& args, int b) {
 // TFLOP/s (K 1035 -> 1250), uniform loads 1172 -> 1233, packed drains + 4 %, persistent tiles over flattened rows
 // 1233 -> 1346, 48-wide tiles 1442.
 template <int S, int N, int MODE>
-__global__ void __launch_bounds__(192, S * N <= 256 ? 2 : 1)
+__global__ void __launch_bounds__(192, ctas_per_sm<S, N>())
     ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                     const __grid_constant__ CUtensorMap mapB2, const TcArgs args) {
     constexpr int A_BYTES = TM * KS * 2;          // 16 KB
@@ -648,10 +658,6 @@ __global__ void __launch_bounds__(192, S * N <= 256 ? 2 : 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(NCOLS));
 }
 
-template <int S, int N>
-size_t tc_smem_bytes() {
-    return (size_t)ring_slots<S, N>() * TM * KS * 2 + 2 * (size_t)S * N * KS * 2 + 1024 + 256;
-}
 
 // ------------------------------------------------------------------------------------------------
 // tensor maps through the driver entry point (no link-time dependence on libcuda)
@@ -697,25 +703,24 @@ long long pipeline_wait_cycles() {
     return (c > 0 && c < WAIT_CYCLES) ? c : WAIT_CYCLES;
 }
 
-// CTAs that the current device holds at once: two per SM where the accumulators leave room for two (the
-// kernel's registers are bounded for it) and the rings fit twice into 228 KB
+// CTAs that the current device holds at once
 template <int S, int N>
 int resident_ctas() {
     int dev = 0, sms = 0;
     DF_CUDA(cudaGetDevice(&dev));
     DF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    return sms * (S * N <= 256 && 2 * (tc_smem_bytes<S, N>() + 1024) <= 228 * 1024 ? 2 : 1);
+    return sms * ctas_per_sm<S, N>();
 }
 
 template <int S, int N, int MODE>
 void launch_tc(cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& b2, const TcArgs& args_in,
                long long total) {
     if (total > INT_MAX - (1 << 20)) throw Error{DF_E_ARG, "tensor-core kernel: too many tiles"};
-    const size_t smem = tc_smem_bytes<S, N>();
+    constexpr int smem = tc_smem_bytes<S, N>();
     TcArgs args = args_in;
     args.wait_cycles = pipeline_wait_cycles();
     args.total = (int)total;
-    DF_CUDA(cudaFuncSetAttribute(ozaki_tc_kernel<S, N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    DF_CUDA(cudaFuncSetAttribute(ozaki_tc_kernel<S, N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const int grid = MODE == 1 ? (int)total : (int)std::min<long long>(total, resident_ctas<S, N>());
     ozaki_tc_kernel<S, N, MODE><<<grid, 192, smem, s>>>(a, b, b2, args);
     DF_CHECK_LAUNCH();
