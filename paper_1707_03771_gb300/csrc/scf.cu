@@ -9,7 +9,8 @@
 // and only the occupied orbitals C_occ = X V_occ are formed each iteration.
 // Every step runs on the device in FP64 (DIIS included); only the energy and max|e| cross to the
 // host each iteration for the convergence test. The symmetric eigensolver is cuSOLVER's dsyevd, for the small
-// matrices of FP64 runs jacobi.cu's.
+// matrices of restricted FP64 runs jacobi.cu's (open-shell runs keep cuSOLVER's at every size: jacobi.cu was not
+// measured there).
 #include <algorithm>
 #include <chrono>
 #include <cstdio>
@@ -452,7 +453,7 @@ class ScfRun {
         DF_CUDA(cudaHostAlloc((void**)&pin_ctl_, sizeof(int) * (2 * DIIS_MAX + 4), cudaHostAllocDefault));
         pin_ctl_[2 * DIIS_MAX + 2] = 0;
         pin_ctl_[2 * DIIS_MAX + 3] = 0;   // the DIIS slot of the iteration being built
-        // per-phase timings take event synchronisations, which stream capture does not allow
+        // no per-phase timings: the build's events could not be read when they are recorded in a captured graph
         saved_sync_timing_ = h_->sync_timing;
         h_->sync_timing = false;
         const char* gv = std::getenv("DFHF_SCF_GRAPHS");
@@ -838,7 +839,7 @@ class ScfRun {
                 DF_CUDA(cudaMalloc((void**)&jac_, sizeof(double) * jacobi_work_doubles(jac_n_)));
             }
             jacobi_eig(s_, m, A, w, A, jac_, info_);
-            orthonormalise(A, m);
+            orthonormalise(A, m, jac_ + (long long)m * m);
             return;
         }
         int lw = 0;
@@ -848,12 +849,13 @@ class ScfRun {
                                    lwork_, info_));
     }
 
-    // rows of V (m x m) orthonormal to rounding: a Newton-Schulz step V <- 1.5 V - 0.5 (V V^T) V, which squares the
-    // error. A Jacobi solve's rotations leave some 1e-14, and vectors that are carried from iteration to iteration add
-    // theirs up: 1.6e-12 after 400 iterations of an SCF that does not converge (n = 200), against 3e-14 from fresh
-    // solves. Scratch: the Jacobi work space, free after a solve.
-    void orthonormalise(double* V, int m) {
-        double *G = jac_, *W = jac_ + (long long)m * m;
+    // rows of V (m x m) orthonormal to rounding, also in W: a Newton-Schulz step V <- 1.5 V - 0.5 (V V^T) V, which
+    // squares the error. A Jacobi solve's rotations leave some 1e-14, and vectors that are carried from iteration to
+    // iteration add theirs up: |C^T S C - 1| was 1.6e-12 after 400 iterations of an SCF that does not converge
+    // (n = 200), now 4.8e-14. 0.1 to 0.4 of 35 ms in an SCF of n = 100. Scratch: the Jacobi work space, free after
+    // a solve.
+    void orthonormalise(double* V, int m, double* W) {
+        double* G = jac_;
         mm(s_, false, true, m, m, m, 1.0, V, m, V, m, 0.0, G, m);
         DF_CUDA(cudaMemcpyAsync(W, V, sizeof(double) * m * m, cudaMemcpyDeviceToDevice, s_));
         mm(s_, false, false, m, m, m, -0.5, G, m, V, m, 1.5, W, m);
@@ -867,15 +869,15 @@ class ScfRun {
         if (!vlast_) {
             DF_CUDA(cudaMalloc((void**)&vlast_, sizeof(double) * 2 * no));
             eig(Fp_, nX_, h_->eps.p);
+            DF_CUDA(cudaMemcpyAsync(vlast_, Fp_, sizeof(double) * no, cudaMemcpyDeviceToDevice, s_));
         } else {
             double* T = vlast_ + no;
             mm(s_, false, false, nX_, nX_, nX_, 1.0, vlast_, nX_, Fp_, nX_, 0.0, T, nX_);
             mm(s_, false, true, nX_, nX_, nX_, 1.0, T, nX_, vlast_, nX_, 0.0, Fp_, nX_);
             jacobi_eig(s_, nX_, Fp_, h_->eps.p, T, jac_, info_);
             mm(s_, false, false, nX_, nX_, nX_, 1.0, T, nX_, vlast_, nX_, 0.0, Fp_, nX_);
-            orthonormalise(Fp_, nX_);
+            orthonormalise(Fp_, nX_, vlast_);
         }
-        DF_CUDA(cudaMemcpyAsync(vlast_, Fp_, sizeof(double) * no, cudaMemcpyDeviceToDevice, s_));
     }
 
     // Fo = X^T Fm X (nX x nX)
