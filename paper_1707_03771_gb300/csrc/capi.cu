@@ -308,7 +308,7 @@ void build_B(df_handle* h, double tau, bool keep, int whitening) {
     DF_CUDA(cudaEventRecord(ev[3], s));
     const char* wenv = std::getenv("DFHF_WHITEN");
     if (whitening == DF_WHITEN_FP64) {
-        // FP64 product on the FP64 pipe, in place by 64-row blocks of L^-1 (a copy first if A is kept)
+        // FP64 product on the FP64 pipe, in place, one launch (a copy first if A is kept)
         if (keep) {
             h->B.ensure(rows);
             DF_CUDA(cudaMemcpyAsync(h->B.p, h->A3c.p, sizeof(double) * rows, cudaMemcpyDeviceToDevice, s));

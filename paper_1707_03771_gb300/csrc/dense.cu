@@ -9,17 +9,18 @@
 // thread-block cluster split the contraction and add their partial tiles through distributed shared memory in a
 // fixed order (deterministic, no workspace); everything that feeds an SCF keeps each element one chain of
 // multiply-adds in ascending order of the contraction, whatever the tile.
-//   - dgemm: general row-major C = alpha op(A) op(B) + beta C (SCF algebra, metric inverse, object operations);
-//     products with one column or one row are matrix-vector kernels bound by HBM.
-//   - dgemm_ordered: the same without a split contraction (metric inverse).
-//   - dgemm_rows: C[b][m][n] = sum_k A[b][m][k] B[k][n] for every batch b at once, any strides.
+//   - dgemm: general row-major C = alpha op(A) op(B) + beta C, never a split contraction (SCF algebra);
+//     dgemm_lower: the same for a lower-triangular B (metric inverse).
+//   - dgemm_rows: C[b][m][n] = sum_k A[b][m][k] B[k][n] for every batch b at once, any strides (object operations,
+//     MP2); its contraction may be split.
+//   - dgemv_rows, dgemv_cols: products with one column or one row (the objects' density contractions), bound by HBM.
 //   - whiten_fp64_inplace: A <- L A for lower-triangular L, in place (the FP64 whitening, paper eq. 1, third
 //     form): one launch, each CTA owning its columns, over the distinct elements mu >= nu only.
 //   - y_transform: Y[mu][P nocc + i] = sum_nu B_{P,mu nu} C_{nu i} reading the packed symmetric B (paper eq. 1,
 //     first form); each stored off-diagonal tile serves both (I,J) and (J,I).
 //   - k_syrk: K = Y Y^T over lower tiles with split partial sums (paper eq. 2, first form), reduced in order.
 // The 64 x 64 register tiles that these kernels replace ran the FP64 pipe at its rate too, but half of it on
-// padding (8 waters: Y 22.7 ms, now 11.4; K 11.9 ms, now 6.3) or on one SM in three (400 x 400 products).
+// padding (8 waters: Y 22.7 ms, now 11.4; K 11.9 ms, now 6.0) or on one SM in three (400 x 400 products).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -60,7 +61,7 @@ struct GemmArgs {
 // C tile of BM = (128 / TX) TM rows by BN = TX TN columns: thread (tx, ty) owns rows ty + TY i and columns
 // tx + TX j; operand steps of 16 k pass through registers into two shared buffers. SYRK: rows = columns = N,
 // B = A, lower tiles only, partial sum `rank` of the contraction into C + rank N N (elements below the diagonal).
-// Bound by the FP64 pipe: at 8 waters (n = 400, naux = 1096, 40 occupied) Y runs at 98 % and K at 90 % of the
+// Bound by the FP64 pipe: at 8 waters (n = 400, naux = 1096, 40 occupied) Y runs at 98 % and K at 94 % of the
 // unit count's 1.256 TFLOP/s on useful work.
 // ------------------------------------------------------------------------------------------------
 template <int TX, int TM, int TN, int AMODE, bool SYRK>
