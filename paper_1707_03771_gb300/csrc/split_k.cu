@@ -788,8 +788,8 @@ int tune_y(df_handle* h, SplitState* st, int nb, float2* Yb) {
     for (int N : {32, 48, 64, 80}) {
         if (seen >= st->cols) break;                 // an earlier width already covers every column
         // over 64 columns or fewer the width divides the occupied width (64): 32 or 64. Over 48 columns a 48-wide tile
-        // takes, against the better of these, 0 to 3 % less (full rows) and 7 % less (packed tiles) of Y's time at 5
-        // slices, and 2 to 6 % more at 3 (350 to 450 functions)
+        // takes, against the better of these, 0 to 4 % (full rows) or 6 to 8 % (packed tiles) less of Y's time at 5
+        // slices, and up to 6 % more at 3 (350 to 450 functions)
         if (N == 48 && st->cols <= 64) continue;
         seen = N;
         const double ms = time_once(h->stream, [&] { y_tc(h, st, S, N, 0, nb, Yb); });
